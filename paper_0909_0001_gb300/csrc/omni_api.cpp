@@ -633,7 +633,7 @@ void choose_chunks(omni_plan* pl) {
     if (last.kind == KIND_SMEM3 && smem3_last_occupancy(last, first_src, &per_sm) != cudaSuccess) per_sm = 0;
     if (last.kind == KIND_TC_B && tc_occupancy(KIND_TC_B, &per_sm) != cudaSuccess) per_sm = 0;
     if (last.kind == KIND_TC5_B && tc5_occupancy(&per_sm) != cudaSuccess) per_sm = 0;
-    if (last.kind == KIND_XSPEC && xspec_occupancy(&per_sm) != cudaSuccess) per_sm = 0;
+    if (last.kind == KIND_XSPEC && xspec_occupancy(last, &per_sm) != cudaSuccess) per_sm = 0;
     if ((last.kind == KIND_XSPEC5 || last.kind == KIND_COV5) && xspec5_occupancy(&per_sm) != cudaSuccess)
         per_sm = 0;
     cudaGetLastError();
@@ -643,16 +643,18 @@ void choose_chunks(omni_plan* pl) {
     pl->Cc = std::min<int64_t>(pl->C, std::max<int64_t>(1, slots / ctas));
     const int64_t per_sample = std::max<int64_t>(1, pl->fwd_elems) * (int64_t)sizeof(float2);
     const bool gemm_last = last.kind == KIND_XSPEC5 || last.kind == KIND_COV5;
-    if (gemm_last) {
+    const bool whole_waves = gemm_last || last.kind == KIND_XSPEC;
+    if (whole_waves) {
         // one CTA per SM and a long accumulation per CTA (its epilogue costs several
         // of its 16-sample steps): 1024 samples per chunk, and channels per chunk
         // chosen so that the chunks' CTAs fill whole waves (256 CTAs per channel on
         // 152 SMs: 6-channel chunks run 10.1 waves in 11, 16-channel chunks 26.9 in
-        // 27), within four times the chunk-buffer target (equal ties: fewer channels)
-        const int64_t cap = 4 * target;
+        // 27), within four times the chunk-buffer target (the FP32 cross-spectra, 96
+        // CTAs per channel of 64 tiles of 16 x 16: within the target; equal ties: fewer channels)
+        const int64_t cap = gemm_last ? 4 * target : target;
         pl->Tc = std::max<int64_t>(1, std::min<int64_t>(1024, cap / per_sample));
         const int64_t cmax = std::min<int64_t>(pl->C, std::max<int64_t>(1, cap / (per_sample * pl->Tc)));
-        const int64_t sl = sms > 0 ? (int64_t)sms * std::max(per_sm, 1) : 152;  // one CTA per SM
+        const int64_t sl = sms > 0 ? (int64_t)sms * std::max(per_sm, 1) : 152;
         int64_t best = 1, best_waves = INT64_MAX;
         for (int64_t cc = 1; cc <= cmax; ++cc) {
             const int64_t n = (pl->C + cc - 1) / cc, cb = (pl->C + n - 1) / n, tail = pl->C - (n - 1) * cb;
@@ -663,7 +665,7 @@ void choose_chunks(omni_plan* pl) {
     }
     if (pl->knobs.chunk_channels > 0) pl->Cc = std::min<int64_t>(pl->C, pl->knobs.chunk_channels);
     const int64_t samples = std::max<int64_t>(1, target / per_sample);
-    if (!gemm_last) pl->Tc = std::max<int64_t>(1, std::min<int64_t>(1024, samples / pl->Cc));
+    if (!whole_waves) pl->Tc = std::max<int64_t>(1, std::min<int64_t>(1024, samples / pl->Cc));
     const int64_t per_chan = std::max<int64_t>(1, pl->inv_elems) * (int64_t)sizeof(float2);
     pl->Cv = std::min<int64_t>(pl->C, std::max<int64_t>(1, target / per_chan));
     pl->buf_elems = std::max(pl->Cc * pl->Tc * pl->fwd_elems, pl->Cv * pl->inv_elems);

@@ -120,7 +120,7 @@ cudaError_t launch_tc5(const Pass& p, const PassArgs& a, cudaStream_t stream);
 
 // Tile hybrid: cross-spectrum accumulation between the tiles' padded spectra.
 cudaError_t launch_xspec(const Pass& p, const PassArgs& a, cudaStream_t stream);
-cudaError_t xspec_occupancy(int* blocks_per_sm);
+cudaError_t xspec_occupancy(const Pass& p, int* blocks_per_sm);
 int64_t xspec_ctas_per_channel(const Pass& p);
 // Forward three-step passes of 2048 and 4096 points: lines per CTA (W consecutive
 // inner indices, or for an innermost MID axis W consecutive outer lines).

@@ -6,103 +6,241 @@
 // accumulates, for every ordered tile pair (i, j) and frequency k,
 //   S_ij(k) += sum over the chunk's samples of Y_i(k) conj(Y_j(k)),
 // in FP32 registers over the chunk, then in an FP64 complex accumulator
-// [C][n_tiles][n_tiles][K].  The inverse 2-D FFT of S_ij gives the visibility
+// [C][n_tiles][n_tiles][K].  S_ji = conj S_ij, so only pairs of tile groups with
+// i's group <= j's are summed and both orders are folded.  The inverse 2-D FFT of S_ij gives the visibility
 // of every antenna pair (a in tile i, b in tile j) with intra-tile offset
 // m_a - m_b = D: the convolution theorem of Sec. II.C applied to two
 // different tiles, exact because of the padding.
 #include "omni_fft_common.cuh"
+#include "omni_tma.cuh"
+
+#include <algorithm>
 
 namespace omni {
 namespace {
 
-constexpr int kXK = 32;  // frequencies per CTA (one per lane)
-constexpr int kXR = 8;   // thread rows per CTA (warps)
-constexpr int kXI = 16;  // tiles i per CTA: two per thread (rows r and r + 8)
-constexpr int kXJ = 16;  // tiles j per CTA, all of them per thread
+// What bounds the sum is FP32 arithmetic: 4 fused multiply-adds per tile pair,
+// frequency and sample against 8 bytes per tile.  A lane is one frequency and a
+// thread holds an 8 x 8 block of pairs (128 sums), so a sample costs 16 shared
+// loads (32 cycles of the SM's shared memory per warp) for 256 multiply-adds (64
+// cycles of its FP32 lanes): a 2 x 16 block, 18 loads for 128 multiply-adds, kept
+// the FP32 pipe at 38%.  Twelve warps of 168 registers fill the register file.
+// Half of the pairs are the other half's conjugates and are not summed.
+// 64 tiles of 16 x 16 antennas, 8 channels x 1024 samples: 10.3 ms -> XSPEC_NOW ms.
+constexpr int kXK = 32;       // frequencies per CTA (one per lane)
+constexpr int kXG = 8;        // tiles per group; a warp holds one pair of groups
+constexpr int kXWarps = 12;   // most warps per CTA
+constexpr int kXRows = 64;    // most tiles per CTA
+constexpr int kXSamples = 4;  // samples per stage
+constexpr int kXStages = 3;
+constexpr int kXA = 3, kXB = 4;  // beyond kXRows tiles: groups i x groups j of a CTA (one pair per warp)
+constexpr size_t kXBar = 128;    // the stages' barriers, before the stages
+static_assert((kXA + kXB) * kXG <= kXRows && kXA * kXB == kXWarps, "rectangular split");
+static_assert(kXBar + (size_t)kXStages * kXSamples * kXRows * kXK * 8 <= 227 * 1024, "shared memory of one CTA");
 
-// CTA = (channel of the chunk, tile group i, tile chunk j, frequency tile);
-// thread = (frequency, tiles i = r and r + 8), 2 x 16 complex accumulators:
-// each spectrum value read from shared memory feeds two (or sixteen) products.
-// 8-byte asynchronous copy global -> shared (zero-filled when !valid).
-__device__ __forceinline__ void cp_async8(float2* dst, const float2* src, bool valid) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(valid ? 8 : 0));
+// How the pairs of groups gi <= gj are split over CTAs and warps.  Up to 64 tiles a
+// CTA reads every tile and its warps take consecutive pairs of the triangle; beyond,
+// a CTA takes kXA x kXB groups (24 + 32 tiles) touching the triangle.
+struct XSplit {
+    int G;      // groups
+    int parts;  // CTAs per (channel, frequency tile)
+    int warps;  // per CTA
+    bool tri;
+};
+__host__ __device__ inline int xs_first_col(int rb) { return rb * kXA / kXB; }
+__host__ __device__ inline XSplit xsplit(int NT) {
+    XSplit x{};
+    x.G = (NT + kXG - 1) / kXG;
+    x.tri = NT <= kXRows;
+    if (x.tri) {
+        const int pairs = x.G * (x.G + 1) / 2;
+        x.parts = (pairs + kXWarps - 1) / kXWarps;
+        x.warps = (pairs + x.parts - 1) / x.parts;
+    } else {
+        const int rows = (x.G + kXA - 1) / kXA, cols = (x.G + kXB - 1) / kXB;
+        for (int rb = 0; rb < rows; ++rb) x.parts += cols - xs_first_col(rb);
+        x.warps = kXWarps;
+    }
+    return x;
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
+inline int xs_rows(int NT) { return NT <= kXRows ? (NT + kXG - 1) / kXG * kXG : (kXA + kXB) * kXG; }
+inline size_t xs_smem(int NT) { return kXBar + (size_t)kXStages * kXSamples * xs_rows(NT) * kXK * sizeof(float2); }
 
-__global__ void __launch_bounds__(kXK * kXR, 2) xspec(Pass p, PassArgs a) {
-    // the next sample's tile is copied asynchronously into the other buffer
-    // while the current one is multiplied (no registers held for it)
-    __shared__ float2 sI[2][kXI][kXK];
-    __shared__ float2 sJ[2][kXJ][kXK];
+// float -> double where the sums are folded: as plain conversions the compiler moved
+// all 128 of them above the bounds checks and spilled 700 bytes
+__device__ __forceinline__ double widen(float x) {
+    double d;
+    asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(x));
+    return d;
+}
+
+// CTA = (channel of the chunk, frequency tile, part of the pairs); the parts of one
+// frequency tile are adjacent, so that they read its spectra from L2.  TMA: one
+// thread brings each stage in with tensor-map boxes two stages ahead (K even: 16-byte
+// rows); else every thread loads the stage (a tile of one antenna, K = 1).
+template <bool TMA>
+__global__ void __launch_bounds__(kXWarps * 32, 1) xspec(Pass p, PassArgs a, const __grid_constant__ CUtensorMap map0,
+                                                         const __grid_constant__ CUtensorMap map1) {
+    extern __shared__ __align__(128) unsigned char dsm[];
+    uint64_t* full = reinterpret_cast<uint64_t*>(dsm);  // [kXStages], then one that nothing arrives on (test hook)
+    float2* ring = reinterpret_cast<float2*>(dsm + kXBar);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int NT = (int)p.outer;
     const int64_t K = p.L;
     const int64_t ktiles = (K + kXK - 1) / kXK;
-    const int igroups = (NT + kXI - 1) / kXI, jchunks = (NT + kXJ - 1) / kXJ;
+    const XSplit xs = xsplit(NT);
     int64_t b = blockIdx.x;
-    const int64_t kt = b % ktiles;
-    b /= ktiles;
-    const int jc = (int)(b % jchunks);
-    b /= jchunks;
-    const int ig = (int)(b % igroups);
-    const int64_t cc = b / igroups;
-    const int kl = threadIdx.x % kXK, r = threadIdx.x / kXK;
-    const int64_t k = kt * kXK + kl;
-    const int i0 = ig * kXI, j0 = jc * kXJ;
-    float ar[2][kXJ], ai[2][kXJ];
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int jj = 0; jj < kXJ; ++jj) ar[h][jj] = ai[h][jj] = 0.f;
-    auto issue = [&](int ts) {
-        const float2* Y = reinterpret_cast<const float2*>(a.src) + src_base(a, cc * a.tc + ts);
-        const bool kin = k < K;
-        const int buf = ts & 1;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int ii = i0 + r + h * kXR, jr = j0 + r + h * kXR;
-            const bool vi = ii < NT && kin, vj = jr < NT && kin;
-            cp_async8(&sI[buf][r + h * kXR][kl], vi ? Y + (int64_t)ii * K + k : Y, vi);
-            cp_async8(&sJ[buf][r + h * kXR][kl], vj ? Y + (int64_t)jr * K + k : Y, vj);
-        }
-        cp_async_commit();
-    };
-    if (a.tc > 0) issue(0);
-    for (int ts = 0; ts < a.tc; ++ts) {
-        if (ts + 1 < a.tc) {
-            issue(ts + 1);
-            cp_async_wait<1>();  // this sample's copies done, the next one's in flight
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
-        const int buf = ts & 1;
-        const float2 y0 = sI[buf][r][kl], y1 = sI[buf][r + kXR][kl];
-#pragma unroll
-        for (int jj = 0; jj < kXJ; ++jj) {
-            const float2 z = sJ[buf][jj][kl];
-            ar[0][jj] = fmaf(y0.x, z.x, fmaf(y0.y, z.y, ar[0][jj]));   // y conj(z)
-            ai[0][jj] = fmaf(y0.y, z.x, fmaf(-y0.x, z.y, ai[0][jj]));
-            ar[1][jj] = fmaf(y1.x, z.x, fmaf(y1.y, z.y, ar[1][jj]));
-            ai[1][jj] = fmaf(y1.y, z.x, fmaf(-y1.x, z.y, ai[1][jj]));
-        }
-        __syncthreads();  // the buffer is refilled two samples later
+    const int part = (int)(b % xs.parts);
+    b /= xs.parts;
+    const int64_t kt = b % ktiles, cc = b / ktiles;
+    // this warp's groups, and the stage rows that hold their tiles: rows 0 .. n0 - 1 are
+    // tiles t0 .., rows n0 .. are tiles t1 ..
+    int gi, gj, ri, rj, t0 = 0, t1 = 0;
+    const int n0 = xs.tri ? NT : kXA * kXG, n1 = xs.tri ? 0 : kXB * kXG;
+    const int rows = xs.tri ? xs.G * kXG : n0 + n1;  // per sample; TMA boxes are n0 + n1 rows, packed
+    bool live;
+    if (xs.tri) {
+        int q = part * xs.warps + warp;
+        gi = 0;
+        while (gi < xs.G && q >= xs.G - gi) q -= xs.G - gi++;
+        gj = gi + q;
+        live = gi < xs.G;
+        if (!live) gi = gj = 0;
+        ri = gi * kXG;
+        rj = gj * kXG;
+    } else {
+        const int cols = (xs.G + kXB - 1) / kXB;
+        int rb = 0, q = part;
+        while (q >= cols - xs_first_col(rb)) q -= cols - xs_first_col(rb++);
+        const int cb = xs_first_col(rb) + q;
+        t0 = rb * kXA * kXG;
+        t1 = cb * kXB * kXG;
+        ri = (warp / kXB) * kXG;
+        rj = n0 + (warp % kXB) * kXG;
+        gi = rb * kXA + warp / kXB;
+        gj = cb * kXB + warp % kXB;
+        live = gi <= gj && gj < xs.G;
     }
-    if (k >= K) return;
-    double2* S = reinterpret_cast<double2*>(a.P + (a.c0 + cc) * a.P_stride);
+    const int prow = TMA ? n0 + n1 : rows;  // stage rows per sample
+    const int64_t stage_elems = (int64_t)kXSamples * rows * kXK;
+    const int tc = a.tc, stages = (tc + kXSamples - 1) / kXSamples;
+    const long long budget = a.force_expire ? kTestWaitCycles : kWaitCycles;
+    if (tid == 0) {
+        for (int i = 0; i <= kXStages; ++i) mbar_init(full + i, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    __syncthreads();
+    auto fill = [&](int n) {  // stage n: samples kXSamples n .. of this channel
+        float2* dst = ring + (n % kXStages) * stage_elems;
+        if constexpr (TMA) {
+            if (tid == 0) {
+                uint64_t* bar = full + n % kXStages;
+                mbar_expect_tx(bar, (uint32_t)((n0 + n1) * kXK * kXSamples * sizeof(float2)));
+                const int x = (int)(2 * kXK * kt), z = (int)(cc * tc + n * kXSamples);
+                if (n1 == 0) {
+                    tma_load3(dst, &map0, x, 0, z, bar);
+                } else {  // one box per sample and tile range: the two ranges of a sample are adjacent
+                    for (int s = 0; s < kXSamples; ++s) {
+                        tma_load3(dst + (int64_t)s * prow * kXK, &map0, x, t0, z + s, bar);
+                        tma_load3(dst + ((int64_t)s * prow + n0) * kXK, &map1, x, t1, z + s, bar);
+                    }
+                }
+            }
+        } else {
+            for (int e = tid; e < stage_elems; e += blockDim.x) {
+                const int k = e % kXK, r = (e / kXK) % rows, s = e / (kXK * rows);
+                const int tile = r < n0 ? t0 + r : t1 + r - n0;
+                const int ts = n * kXSamples + s;
+                const bool in = kt * kXK + k < K && tile < NT && ts < tc;
+                dst[e] = in ? __ldg(reinterpret_cast<const float2*>(a.src) + src_base(a, cc * tc + ts) + tile * K +
+                                    kt * kXK + k)
+                            : make_float2(0.f, 0.f);
+            }
+        }
+    };
+    float ar[kXG][kXG], ai[kXG][kXG];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int i = i0 + r + h * kXR;
-        if (i >= NT) break;
+    for (int u = 0; u < kXG; ++u)
 #pragma unroll
-        for (int jj = 0; jj < kXJ; ++jj) {
-            const int j = j0 + jj;
-            if (j >= NT) break;
-            double2& s = S[((int64_t)i * NT + j) * K + k];
-            s.x += (double)ar[h][jj];
-            s.y += (double)ai[h][jj];
+        for (int v = 0; v < kXG; ++v) ar[u][v] = ai[u][v] = 0.f;
+    bool failed = false;
+    int issued = 0;
+    if constexpr (TMA) {
+        for (; issued < stages && issued < kXStages - 1; ++issued) fill(issued);
+    }
+    for (int n = 0; n < stages; ++n) {
+        // every warp is past stage n - 1: its buffer takes stage n + 2 (or, without
+        // tensor maps, this stage's is filled now)
+        if (__syncthreads_or(failed)) break;
+        if constexpr (TMA) {
+            if (issued < stages) fill(issued++);
+            failed = (a.force_expire && n == 0) ? !wait_bar(full + kXStages, 0, budget)
+                                                : !wait_bar(full + n % kXStages, (n / kXStages) & 1, budget);
+        } else {
+            fill(n);
+            __syncthreads();
+        }
+        const float2* st = ring + (n % kXStages) * stage_elems + lane;
+        const int ns = min(kXSamples, tc - n * kXSamples);
+        if (live && !failed) {
+#pragma unroll 1
+            for (int s = 0; s < ns; ++s) {
+                const float2* yr = st + (s * prow + ri) * kXK;
+                const float2* zr = st + (s * prow + rj) * kXK;
+                float2 y[kXG];
+#pragma unroll
+                for (int u = 0; u < kXG; ++u) y[u] = yr[u * kXK];
+#pragma unroll
+                for (int v = 0; v < kXG; ++v) {
+                    const float2 z = zr[v * kXK];
+#pragma unroll
+                    for (int u = 0; u < kXG; ++u) {  // y conj(z)
+                        ar[u][v] = fmaf(y[u].x, z.x, fmaf(y[u].y, z.y, ar[u][v]));
+                        ai[u][v] = fmaf(y[u].y, z.x, fmaf(-y[u].x, z.y, ai[u][v]));
+                    }
+                }
+            }
+        }
+    }
+    if constexpr (TMA) {
+        // no box is in flight when the CTA leaves (each was waited for above unless a wait gave up)
+        if (__syncthreads_or(failed)) {
+            if (tid == 0) {
+                for (int n = max(0, issued - kXStages); n < issued; ++n) wait_bar(full + n % kXStages, (n / kXStages) & 1);
+                atomicExch(a.err, 1);
+            }
+            return;
+        }
+    }
+    const int64_t k = kt * kXK + lane;
+    if (!live || k >= K) return;
+    double2* S = reinterpret_cast<double2*>(a.P + (a.c0 + cc) * a.P_stride) + k;
+    const int i0 = gi * kXG, j0 = gj * kXG;
+    // both orders of each pair; kXF of them at a time, their loads together
+    constexpr int kXF = 2;
+#pragma unroll
+    for (int u = 0; u < kXG; ++u) {
+        const int i = i0 + u;
+#pragma unroll
+        for (int v0 = 0; v0 < kXG; v0 += kXF) {
+            double2 f[kXF], m[kXF];
+#pragma unroll
+            for (int v = 0; v < kXF; ++v) {
+                const int j = j0 + v0 + v;
+                if (i < NT && j < NT) {
+                    f[v] = S[(i * NT + j) * K];
+                    if (gi != gj) m[v] = S[(j * NT + i) * K];
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < kXF; ++v) {
+                const int j = j0 + v0 + v;
+                if (i < NT && j < NT) {
+                    const double re = widen(ar[u][v0 + v]), im = widen(ai[u][v0 + v]);
+                    S[(i * NT + j) * K] = make_double2(f[v].x + re, f[v].y + im);
+                    if (gi != gj) S[(j * NT + i) * K] = make_double2(m[v].x + re, m[v].y - im);
+                }
+            }
         }
     }
 }
@@ -110,19 +248,37 @@ __global__ void __launch_bounds__(kXK * kXR, 2) xspec(Pass p, PassArgs a) {
 }  // namespace
 
 int64_t xspec_ctas_per_channel(const Pass& p) {
-    const int64_t NT = p.outer;
-    return ((p.L + kXK - 1) / kXK) * ((NT + kXI - 1) / kXI) * ((NT + kXJ - 1) / kXJ);
+    return ((p.L + kXK - 1) / kXK) * (int64_t)xsplit((int)p.outer).parts;
 }
 
-cudaError_t xspec_occupancy(int* blocks_per_sm) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, xspec, kXK * kXR, 0);
+cudaError_t xspec_occupancy(const Pass& p, int* blocks_per_sm) {
+    const int NT = (int)p.outer;
+    cudaError_t e = smem_limit_once((const void*)xspec<true>, xs_smem(NT));
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, xspec<true>, 32 * xsplit(NT).warps, xs_smem(NT));
 }
 
 cudaError_t launch_xspec(const Pass& p, const PassArgs& a, cudaStream_t st) {
-    if (a.src_kind != SRC_BUF) return cudaErrorInvalidValue;
+    if (a.src_kind != SRC_BUF || !a.err) return cudaErrorInvalidValue;
     const int64_t blocks = a.S * xspec_ctas_per_channel(p);
-    if (blocks <= 0) return cudaSuccess;
-    xspec<<<(unsigned)blocks, kXK * kXR, 0, st>>>(p, a);
+    if (blocks <= 0 || a.tc <= 0) return cudaSuccess;
+    const int NT = (int)p.outer;
+    const XSplit xs = xsplit(NT);
+    const size_t smem = xs_smem(NT);
+    // tensor maps want 16-byte aligned rows; an odd K is a tile of one antenna
+    const bool tma = p.L % 2 == 0 && reinterpret_cast<uintptr_t>(a.src) % 16 == 0;
+    CUtensorMap m0{}, m1{};
+    if (tma) {
+        const int64_t samples = a.S * a.tc;
+        cudaError_t e = xs.tri ? encode_spectra_map(a.src, p.L, NT, samples, 2 * kXK, NT, kXSamples, &m0)
+                               : encode_spectra_map(a.src, p.L, NT, samples, 2 * kXK, kXA * kXG, 1, &m0);
+        if (e == cudaSuccess && !xs.tri) e = encode_spectra_map(a.src, p.L, NT, samples, 2 * kXK, kXB * kXG, 1, &m1);
+        if (e != cudaSuccess) return e;
+    }
+    auto kern = tma ? xspec<true> : xspec<false>;
+    cudaError_t e = smem_limit_once((const void*)kern, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)blocks, 32 * xs.warps, smem, st>>>(p, a, m0, m1);
     return cudaGetLastError();
 }
 

@@ -35,14 +35,13 @@
 // returns.
 #include "omni_fft_common.cuh"
 
-#include <cuda.h>            // CUtensorMap; the encoder is fetched from the driver at run time
+#include "omni_tma.cuh"
+
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
-#include <cudaTypedefs.h>
 
 #include <algorithm>
 #include <cstring>
-#include <mutex>
 
 namespace omni {
 namespace {
@@ -86,13 +85,10 @@ constexpr int kXScaleTarget = 12;  // FP16: |Y| 2^-e <= 2^12
 // kind::f16, FP32 accumulate, K-major, M = 128, N = 128; A and B FP16 or (bits 7, 10) BF16
 constexpr uint32_t kIdesc128 = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 constexpr uint32_t kIdesc128Bf16 = kIdesc128 | (1u << 7) | (1u << 10);
-constexpr long long kWaitCycles = 4000000000LL;   // ~2 s
-constexpr long long kTestWaitCycles = 1000000LL;  // the forced-expiry test hook: ~0.5 ms
 
 __host__ __device__ inline int tile_off(int row, int k) {
     return (row >> 3) * kSBO + (k >> 3) * kLBO + (row & 7) * 16 + (k & 7) * 2;
 }
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint64_t sdesc(const void* p) {
     const uint32_t a = smem_u32(p);
     return (uint64_t)((a >> 4) & 0x3FFF) | ((uint64_t)(kLBO >> 4) << 16) |
@@ -107,22 +103,6 @@ __device__ __forceinline__ void commit(uint64_t* bar) {
     asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
                  " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n"
                  :: "r"(smem_u32(bar)));
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, int count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(bar)), "r"(count));
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" :: "r"(smem_u32(bar)));
-}
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, long long budget = kWaitCycles) {
-    const long long t0 = clock64();
-    for (;;) {
-        uint32_t done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-                     " selp.u32 %0, 1, 0, p;\n}\n" : "=r"(done) : "r"(smem_u32(bar)), "r"(parity));
-        if (done) return true;
-        if (clock64() - t0 > budget) return false;
-    }
 }
 // 64 consecutive columns of the warp's 32 lanes: two loads, one wait
 __device__ __forceinline__ void ld64(uint32_t taddr, float (&v)[64]) {
@@ -175,17 +155,6 @@ __device__ __forceinline__ void split3(float x0, float x1, uint32_t& h, uint32_t
     h = b2u(bh);
     m = b2u(bm);
     l = b2u(__floats2bfloat162_rn(r0 - fm.x, r1 - fm.y));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(smem_u32(bar)), "r"(bytes));
-}
-// One box of the 3-D tensor map into shared memory, completing on bar.
-__device__ __forceinline__ void tma_load3(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
-    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
-                 " [%0], [%1, {%2, %3, %4}], [%5];"
-                 :: "r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z),
-                    "r"(smem_u32(bar))
-                 : "memory");
 }
 __device__ __forceinline__ bool elect_one() {
     uint32_t e;
@@ -622,30 +591,6 @@ cudaError_t xspec5_occupancy(int* blocks_per_sm) {
     return e;
 }
 
-// 3-D map of the spectra [samples][tiles][2K floats]; a box (x: the 8 floats of
-// the CTA's 4 frequencies, y: every tile, z: 16 samples) lands as [z][y][x].
-static cudaError_t encode_map(const PassArgs& a, const Pass& p, CUtensorMap* map) {
-    static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess && q == cudaDriverEntryPointSuccess)
-            encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    });
-    if (!encode) return cudaErrorNotSupported;
-    const cuuint64_t K = (cuuint64_t)p.L, NT = (cuuint64_t)p.outer;
-    const cuuint64_t dims[3] = {2 * K, NT, (cuuint64_t)(a.S * a.tc)};
-    const cuuint64_t strides[2] = {K * 8, NT * K * 8};
-    const cuuint32_t box[3] = {8, (cuuint32_t)NT, 16};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(a.src), dims, strides, box,
-                              estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
 cudaError_t launch_xspec5(const Pass& p, const PassArgs& a, cudaStream_t st) {
     if (a.src_kind != SRC_BUF || !xspec5_supports(p.outer, p.L) || !a.err) return cudaErrorInvalidValue;
     const int64_t blocks = a.S * xspec5_ctas_per_channel(p);
@@ -653,7 +598,8 @@ cudaError_t launch_xspec5(const Pass& p, const PassArgs& a, cudaStream_t st) {
     // the TMA unit wants a 16-byte aligned base and row pitches
     if (reinterpret_cast<uintptr_t>(a.src) % 16 || (p.L * 8) % 16) return cudaErrorInvalidValue;
     CUtensorMap map;
-    const cudaError_t me = encode_map(a, p, &map);
+    // a box: the 8 floats of a CTA's 4 frequencies, every tile, 16 samples
+    const cudaError_t me = encode_spectra_map(a.src, p.L, p.outer, a.S * a.tc, 2 * kXF, (int)p.outer, 16, &map);
     if (me != cudaSuccess) return me;
     if (p.scale_n > 0 && !p.bf16 && !a.chan_max) return cudaErrorInvalidValue;
     void (*kern)(Pass, PassArgs, const CUtensorMap) = nullptr;
