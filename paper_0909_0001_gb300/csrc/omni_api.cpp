@@ -1348,8 +1348,7 @@ omni_status omni_fengine(const int8_t* raw_dev, int64_t n_antennas, int64_t n_sa
         return fail(OMNI_ERR_INVALID_ARG, "launch too large: split the antennas or the samples");
     cudaError_t e = launch_fengine(raw_dev, n_antennas, n_samples, n_channels, taps, window_dev,
                                    reinterpret_cast<const float2*>(gains_dev), scale,
-                                   out_dtype == OMNI_IN_CI8, out_dev, reinterpret_cast<float2*>(scratch_dev),
-                                   (cudaStream_t)stream);
+                                   out_dtype == OMNI_IN_CI8, out_dev, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "F-engine launch");
     return OMNI_OK;
 }

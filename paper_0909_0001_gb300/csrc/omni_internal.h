@@ -141,15 +141,14 @@ cudaError_t launch_chan_absmax(const void* volts, int src_kind, int64_t vc0, int
 cudaError_t launch_xspec5_transpose(const double* P, int64_t P_stride, int64_t cv, int64_t K, int64_t NP,
                                     float2* dst, cudaStream_t stream);
 
-// F-engine: frames per antenna, scratch bytes, CTAs of the largest launch, and
-// the launches (fused for F <= 256; else spectra into scratch [N][T][F], then
-// calibrated, quantised or not, transposed to [F][T][N]).
+// F-engine: frames per antenna, the scratch a caller provides, the CTA count that a
+// launch may not exceed, and the launch (one pass from samples to [F][T][N]).
 int64_t fengine_frames(int64_t n_samples, int32_t F, int32_t P);
 int64_t fengine_scratch_bytes(int64_t N, int64_t S, int32_t F, int32_t P);
-int64_t fengine_ctas(int64_t N, int64_t T, int32_t F);  // largest launch, CTAs
+int64_t fengine_ctas(int64_t N, int64_t T, int32_t F);
 cudaError_t launch_fengine(const int8_t* raw, int64_t N, int64_t S, int32_t F, int32_t P,
                            const float* window, const float2* gains, float scale, int out_i8,
-                           void* out, float2* scratch, cudaStream_t stream);
+                           void* out, cudaStream_t st);
 
 // Set the calling thread's omni_last_error() message.
 void set_last_error(const char* msg);
