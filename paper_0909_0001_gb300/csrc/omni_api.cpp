@@ -650,16 +650,19 @@ void choose_chunks(omni_plan* pl) {
         // chosen so that the chunks' CTAs fill whole waves (256 CTAs per channel on
         // 152 SMs: 6-channel chunks run 10.1 waves in 11, 16-channel chunks 26.9 in
         // 27), within four times the chunk-buffer target (the FP32 cross-spectra, 96
-        // CTAs per channel of 64 tiles of 16 x 16: within the target; equal ties: fewer channels)
+        // CTAs per channel of 64 tiles of 16 x 16: within the target)
         const int64_t cap = gemm_last ? 4 * target : target;
         pl->Tc = std::max<int64_t>(1, std::min<int64_t>(1024, cap / per_sample));
         const int64_t cmax = std::min<int64_t>(pl->C, std::max<int64_t>(1, cap / (per_sample * pl->Tc)));
         const int64_t sl = sms > 0 ? (int64_t)sms * std::max(per_sm, 1) : 152;
-        int64_t best = 1, best_waves = INT64_MAX;
+        // a chunk's launches, gaps and ramps cost about a quarter of a wave (50 tiles of 12 x 12
+        // antennas, 16 channels x 500 samples: 16 one-channel chunks 4.3 ms, one chunk 3.6)
+        int64_t best = 1, best_cost = INT64_MAX;
         for (int64_t cc = 1; cc <= cmax; ++cc) {
             const int64_t n = (pl->C + cc - 1) / cc, cb = (pl->C + n - 1) / n, tail = pl->C - (n - 1) * cb;
             const int64_t waves = (n - 1) * ((cb * ctas + sl - 1) / sl) + (tail * ctas + sl - 1) / sl;
-            if (waves < best_waves) best = cc, best_waves = waves;
+            const int64_t cost = 4 * waves + n;
+            if (cost < best_cost) best = cc, best_cost = cost;
         }
         pl->Cc = best;
     }

@@ -619,29 +619,38 @@ cudaError_t launch_xspec5(const Pass& p, const PassArgs& a, cudaStream_t st) {
 
 namespace {
 // one CTA per (channel, slice of its samples); block max in shared memory, then
-// one atomicMax per CTA on the float's bits (non-negative floats order as integers)
+// one atomicMax per CTA on the float's bits (non-negative floats order as integers).
+// A channel's samples of the chunk are one run of memory, read 16 bytes at a time
+// between its unaligned ends.
 template <int SRC>
 __global__ void __launch_bounds__(256) chan_absmax(const void* volts, int64_t vc0, int64_t T, int64_t t0, int64_t N,
                                                    int64_t tc, float* out) {
     __shared__ float red[8];
     const int64_t c = blockIdx.y;
-    const int64_t per = tc * N;  // complex values of the channel in the chunk
+    using S = typename std::conditional<SRC == SRC_CI8, int8_t, float>::type;
+    constexpr int PER = 16 / sizeof(S);
+    const S* run = reinterpret_cast<const S*>(volts) + 2 * ((vc0 + c) * T + t0) * N;
+    const int64_t n = 2 * tc * N;  // real values
+    const int64_t head = min(n, (int64_t)(((16 - ((uintptr_t)run & 15)) & 15) / sizeof(S)));
+    const int64_t quads = (n - head) / PER;
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, all = (int64_t)gridDim.x * blockDim.x;
     float m = 0.f;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < per; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = i / N, n = i - t * N;
-        const int64_t e = ((vc0 + c) * T + t0 + t) * N + n;
-        float re, im;
-        if (SRC == SRC_CI8) {
-            const char2 v = reinterpret_cast<const char2*>(volts)[e];
-            re = (float)v.x;
-            im = (float)v.y;
-        } else {
-            const float2 v = reinterpret_cast<const float2*>(volts)[e];
-            re = v.x;
-            im = v.y;
+#pragma unroll 4
+    for (int64_t i = first; i < quads; i += all) {
+        const uint4 q = __ldg(reinterpret_cast<const uint4*>(run + head) + i);
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if constexpr (SRC == SRC_CI8) {
+#pragma unroll
+                for (int b = 0; b < 4; ++b) m = fmaxf(m, fabsf((float)(int8_t)(w[k] >> (8 * b))));
+            } else {
+                m = fmaxf(m, fabsf(__uint_as_float(w[k])));
+            }
         }
-        m = fmaxf(m, fmaxf(fabsf(re), fabsf(im)));
     }
+    for (int64_t i = first; i < n - PER * quads; i += all)  // the ends
+        m = fmaxf(m, fabsf((float)run[i < head ? i : PER * quads + i]));
     for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
     __syncthreads();
@@ -660,7 +669,8 @@ cudaError_t launch_chan_absmax(const void* volts, int src_kind, int64_t vc0, int
     cudaError_t e = cudaMemsetAsync(out, 0, (size_t)cc * sizeof(float), st);
     if (e != cudaSuccess || tc <= 0 || N <= 0) return e;
     const int64_t per = tc * N;
-    const unsigned bx = (unsigned)std::min<int64_t>(64, (per + 255) / 256);
+    // eight CTAs per SM over all channels, at least 64 for each
+    const unsigned bx = (unsigned)std::min<int64_t>(std::max<int64_t>(64, 8 * 152 / cc), (per + 255) / 256);
     const dim3 grid(bx, (unsigned)cc);
     if (src_kind == SRC_CI8)
         chan_absmax<SRC_CI8><<<grid, 256, 0, st>>>(volts, vc0, T, t0, N, tc, out);
