@@ -252,6 +252,8 @@ struct omni_plan {
     omni_precision precision = OMNI_FP32;
     std::vector<Pass> fwd, inv;
     int64_t Cc = 1, Tc = 1;   // forward chunk: channels x samples
+    int slices = 1;           // LAST: slices of a chunk's samples (fewer CTAs than the GPU holds)
+    float* part = nullptr;    // ... their sums, [slices][Cc][L]
     bool beams = false;       // beam-space plan: level-1 axes unpadded, no lag over them
     int64_t n_tiles = 0;      // tile-hybrid plan: identical tiles at arbitrary offsets
     int64_t lag_pairs = 0;    // mixed 2-level plan with a lag-sum level 2: coarse lags kept per
@@ -350,11 +352,12 @@ int elem_bytes(omni_dtype t) { return t == OMNI_IN_CI8 ? 2 : 8; }
 // Level pass tiling (fixed at compile time in the kernels): the finest level
 // (inner == 1) packs whole blocks, W = 1; a coarser level takes W consecutive
 // inner indices, W = 256 * LPT / L with LPT = 2 lines per thread (1 for
-// 64-point axes) in a LAST pass and 1 in a MID pass.
+// 64-point axes) in a LAST pass and 1 in a MID pass, or the two-column LAST pass's own.
 void choose_level(Pass& p) {
     p.kind = KIND_LEVEL;
     const int lpt = p.mode == MODE_LAST ? (p.L >= 64 ? 1 : 2) : 1;
     p.W = p.inner == 1 ? 1 : 256 * lpt / p.L;
+    if (p.mode == MODE_LAST && level_last_columns(p.L, p.inner) > 0) p.W = level_last_columns(p.L, p.inner);
 }
 
 // Passes of 2048 and 4096 points: the three-step kernel (16-point register
@@ -399,7 +402,7 @@ omni_status build_passes(omni_plan* pl) {
         const int d = axes[a];
         const bool pair = use_level && (d % 2 == 0) && a + 1 < axes.size() && axes[a + 1] == d + 1 &&
                           g.Lp[d] == g.Lp[d + 1] && is_pow2(g.Lp[d]) && g.Lp[d] <= 64 &&
-                          !(pl->beams && d < 2);
+                          !(pl->beams && d < 2 && (g.Lp[d] > 32 || g.Lp[d] < 4));
         stages.push_back({d, pair});
         if (pair) ++a;
     }
@@ -669,6 +672,19 @@ void choose_chunks(omni_plan* pl) {
     if (pl->knobs.chunk_channels > 0) pl->Cc = std::min<int64_t>(pl->C, pl->knobs.chunk_channels);
     const int64_t samples = std::max<int64_t>(1, target / per_sample);
     if (!whole_waves) pl->Tc = std::max<int64_t>(1, std::min<int64_t>(1024, samples / pl->Cc));
+    // too few CTAs for the GPU: cut the samples into slices, the number that takes the
+    // least time in whole waves (a slice's fold counts as a 50th of the pass), within 256 MB of sums
+    pl->slices = 1;
+    if (last.kind == KIND_LEVEL || last.kind == KIND_REG || last.kind == KIND_SMEM || last.kind == KIND_SMEM3 ||
+        last.kind == KIND_DIRECT) {
+        const int64_t c = last.kind == KIND_DIRECT ? pl->Cc * ((last.inner + 63) / 64) : pl->Cc * ctas;
+        const int64_t most = std::min<int64_t>((int64_t)64, ((int64_t)256 << 20) / std::max<int64_t>(1, 4 * pl->Cc * acc_doubles(pl)));
+        double best = 1.0 * ceil_div(c, slots);
+        for (int64_t k = 2; k <= most && c < 2 * slots; ++k) {
+            const double t = (double)ceil_div(c * k, slots) / k + 0.02;
+            if (t < 0.9 * best) best = t, pl->slices = (int)k;
+        }
+    }
     const int64_t per_chan = std::max<int64_t>(1, pl->inv_elems) * (int64_t)sizeof(float2);
     pl->Cv = std::min<int64_t>(pl->C, std::max<int64_t>(1, target / per_chan));
     pl->buf_elems = std::max(pl->Cc * pl->Tc * pl->fwd_elems, pl->Cv * pl->inv_elems);
@@ -697,6 +713,7 @@ void release(omni_plan* pl) {
     cudaFree(pl->buf[0]);
     cudaFree(pl->buf[1]);
     cudaFree(pl->chan_max);
+    cudaFree(pl->part);
     cudaFree(pl->P);
     cudaFree(pl->dev_err);
     cudaFree(pl->vis_tmp);
@@ -891,6 +908,8 @@ omni_status run_chunk(omni_plan* pl, const void* volts, int64_t vc0, int64_t Tsr
         }
         if (p.mode == MODE_LAST) {
             a.S = cc;
+            a.split = (int)std::min<int64_t>(pl->slices, tc);
+            a.part = pl->part;
         } else {
             a.S = cc * tc;
             a.dst = dst;
@@ -904,6 +923,7 @@ omni_status run_chunk(omni_plan* pl, const void* volts, int64_t vc0, int64_t Tsr
             const int64_t cc_tc = cc - cc_split;
             PassArgs b = a;
             b.S = cc_split;
+            b.split = 1;
             b.c0 = c0 + cc_tc;
             b.src = (const float2*)src + cc_tc * tc * src_stride;
             // the tensor-core first pass scales the spectra by 1/16, the FP32 one does not
@@ -916,6 +936,7 @@ omni_status run_chunk(omni_plan* pl, const void* volts, int64_t vc0, int64_t Tsr
             OMNI_CUDA(cudaEventRecord(pl->split_done[slot], pl->split_stream), "cudaEventRecord");
         }
         cudaError_t e = launch_counted(pl, (int)k, p, a, launch_stream);
+        if (e == cudaSuccess && p.mode == MODE_LAST) e = launch_fold_parts(a, launch_stream);
         if (e != cudaSuccess) return cuda_fail(e, "forward pass launch");
         if (cc_split > 0)
             OMNI_CUDA(cudaStreamWaitEvent(st, pl->split_done[slot], 0), "cudaStreamWaitEvent");
@@ -1496,6 +1517,11 @@ static omni_status create_plan(const omni_level* levels, int n_levels, int64_t n
     bool data_scale = false;
     for (const Pass& q : pl->fwd) data_scale = data_scale || (q.scale_n > 0 && !q.bf16);
     if (data_scale && (e = cudaMalloc(&pl->chan_max, (size_t)2 * pl->Cc * sizeof(float))) != cudaSuccess) {
+        release(pl);
+        return cuda_fail(e, "cudaMalloc");
+    }
+    if (pl->slices > 1 &&
+        (e = cudaMalloc(&pl->part, (size_t)pl->slices * pl->Cc * acc_doubles(pl) * sizeof(float))) != cudaSuccess) {
         release(pl);
         return cuda_fail(e, "cudaMalloc");
     }

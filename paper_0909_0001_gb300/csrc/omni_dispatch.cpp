@@ -15,11 +15,11 @@ cudaError_t launch_smem_c(const Pass& p, const PassArgs& a, cudaStream_t st);
 cudaError_t launch_direct(const Pass& p, const PassArgs& a, cudaStream_t st);
 cudaError_t launch_level_a(const Pass& p, const PassArgs& a, cudaStream_t st);
 cudaError_t launch_level_b(const Pass& p, const PassArgs& a, cudaStream_t st);
-cudaError_t level_occupancy_a(int L, bool finest, int src_kind, int* out);
+cudaError_t level_occupancy_a(int L, int64_t inner, int src_kind, int* out);
 cudaError_t smem_last_occupancy_a(const Pass& p, int src_kind, int* blocks_per_sm);
 cudaError_t smem_last_occupancy_b(const Pass& p, int src_kind, int* blocks_per_sm);
 cudaError_t smem_last_occupancy_c(const Pass& p, int src_kind, int* blocks_per_sm);
-cudaError_t level_occupancy_b(int L, bool finest, int src_kind, int* out);
+cudaError_t level_occupancy_b(int L, int64_t inner, int src_kind, int* out);
 cudaError_t level_stream_occupancy_a(int L, int src_kind, int* out);
 cudaError_t level_stream_occupancy_b(int L, int src_kind, int* out);
 cudaError_t upload_twiddles_reg_a();
@@ -56,8 +56,8 @@ cudaError_t smem_last_occupancy(const Pass& p, int src_kind, int* blocks_per_sm)
 }
 
 cudaError_t level_last_occupancy(const Pass& p, int src_kind, int* blocks_per_sm) {
-    return p.L <= 16 ? level_occupancy_a(p.L, p.inner == 1, src_kind, blocks_per_sm)
-                     : level_occupancy_b(p.L, p.inner == 1, src_kind, blocks_per_sm);
+    return p.L <= 16 ? level_occupancy_a(p.L, p.inner, src_kind, blocks_per_sm)
+                     : level_occupancy_b(p.L, p.inner, src_kind, blocks_per_sm);
 }
 
 cudaError_t level_stream_occupancy(const Pass& p, int src_kind, int* blocks_per_sm) {

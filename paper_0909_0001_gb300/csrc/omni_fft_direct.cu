@@ -26,7 +26,9 @@ __global__ void __launch_bounds__(256) pass_direct(Pass p, PassArgs a) {
         const int k = (int)(r / inner);
         const int64_t i = r - (int64_t)k * inner;
         float acc = 0.0f;
-        for (int tt = 0; tt < a.tc; ++tt) {
+        int tb, te;
+        slice_samples(a, tb, te);
+        for (int tt = tb; tt < te; ++tt) {
             const int64_t base = src_base(a, cc * a.tc + tt) + i;
             float2 sum = make_float2(0.f, 0.f);
             int m = 0;
@@ -40,7 +42,7 @@ __global__ void __launch_bounds__(256) pass_direct(Pass p, PassArgs a) {
             }
             acc += cnorm(sum);
         }
-        a.P[(a.c0 + cc) * a.P_stride + (int64_t)k * inner + i] += (double)acc;
+        fold_last(a, cc, (int64_t)k * inner + i, acc);
     } else {
         const int64_t per = p.outer * (int64_t)Q * inner;
         if (flat >= a.S * per) return;
@@ -160,7 +162,7 @@ __global__ void __launch_bounds__(256, 3) pass_dft(Pass p, PassArgs a) {
         if (s < a.S) {
             if constexpr (MODE == MODE_LAST) {
                 src = src_base(a, s * a.tc) + r;
-                dst = (a.c0 + s) * a.P_stride + r;
+                dst = g;  // split into channel and column again at the fold
             } else {
                 const int64_t o = r / inner, i = r - o * inner;
                 src = src_base(a, s) + o * (int64_t)n * inner + i;
@@ -176,13 +178,14 @@ __global__ void __launch_bounds__(256, 3) pass_dft(Pass p, PassArgs a) {
     const int64_t step = a.src_kind == SRC_BUF ? a.src_stride : a.N;  // LAST: from sample to sample
 
     float acc[MODE == MODE_LAST ? KB * OUTS : 1];  // LAST: |X|^2 over the samples (LN = 1, one group per pass)
-    const int n_samples = MODE == MODE_LAST ? a.tc : 1;
+    int tb = 0, te = 1;
+    if constexpr (MODE == MODE_LAST) slice_samples(a, tb, te);
     const int passes = (d.groups + d.kg - 1) / d.kg;
     for (int ps = 0; ps < (MODE == MODE_LAST ? passes : 1); ++ps) {
         if constexpr (MODE == MODE_LAST)
 #pragma unroll
             for (int e = 0; e < KB * OUTS; ++e) acc[e] = 0.f;
-        for (int ts = 0; ts < n_samples; ++ts) {
+        for (int ts = tb; ts < te; ++ts) {
             // load: terms of one line along memory (contiguous lines), or one term of many lines
             const bool along = inner == 1;
             const int jmax = along ? d.rows : d.lines, dj = blockDim.x % jmax, dl = blockDim.x / jmax;
@@ -311,6 +314,7 @@ __global__ void __launch_bounds__(256, 3) pass_dft(Pass p, PassArgs a) {
         if constexpr (MODE == MODE_LAST) {
             const int g = g0 + ps * d.kg;
             if (g < d.groups && db[lx] >= 0) {
+                const int64_t cc = db[lx] / inner, i = db[lx] - cc * inner;
 #pragma unroll
                 for (int b = 0; b < KB; ++b) {
                     const int r = g * KB + b;
@@ -319,8 +323,8 @@ __global__ void __launch_bounds__(256, 3) pass_dft(Pass p, PassArgs a) {
                     for (int h = 0; h < 2; ++h) {
                         if (h && 2 * r == n) continue;
                         const int k = h ? r + n : r, m = h ? n - r : (r ? L - r : 0);
-                        a.P[db[lx] + (int64_t)k * inner] += (double)acc[b * OUTS + 2 * h];
-                        if (m != k) a.P[db[lx] + (int64_t)m * inner] += (double)acc[b * OUTS + 2 * h + 1];
+                        fold_last(a, cc, (int64_t)k * inner + i, acc[b * OUTS + 2 * h]);
+                        if (m != k) fold_last(a, cc, (int64_t)m * inner + i, acc[b * OUTS + 2 * h + 1]);
                     }
                 }
             }
@@ -356,7 +360,8 @@ cudaError_t launch_dft_t(const Pass& p, const PassArgs& a, cudaStream_t st) {
     auto k = pass_dft<MODE, SRC, HALF>;
     cudaError_t e = smem_limit_once((const void*)k, d.smem);
     if (e != cudaSuccess) return e;
-    k<<<(unsigned)((lines + d.lines - 1) / d.lines), d.threads, d.smem, st>>>(p, a);
+    const int64_t blocks = (lines + d.lines - 1) / d.lines;
+    k<<<MODE == MODE_LAST ? last_grid(blocks, a) : dim3((unsigned)blocks), d.threads, d.smem, st>>>(p, a);
     return cudaGetLastError();
 }
 
@@ -376,7 +381,7 @@ cudaError_t launch_direct_t(const Pass& p, const PassArgs& a, cudaStream_t st) {
     }
     const int threads = 256;
     const int64_t blocks = (work + threads - 1) / threads;
-    pass_direct<MODE, SRC><<<(unsigned)blocks, threads, 0, st>>>(p, a);
+    pass_direct<MODE, SRC><<<MODE == MODE_LAST ? last_grid(blocks, a) : dim3((unsigned)blocks), threads, 0, st>>>(p, a);
     return cudaGetLastError();
 }
 

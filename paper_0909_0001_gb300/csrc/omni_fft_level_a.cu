@@ -12,11 +12,11 @@ cudaError_t launch_level_a(const Pass& p, const PassArgs& a, cudaStream_t st) {
     }
 }
 
-cudaError_t level_occupancy_a(int L, bool finest, int src_kind, int* out) {
+cudaError_t level_occupancy_a(int L, int64_t inner, int src_kind, int* out) {
     switch (L) {
-        case 4: return level_last_blocks_per_sm<4>(finest, src_kind, out);
-        case 8: return level_last_blocks_per_sm<8>(finest, src_kind, out);
-        case 16: return level_last_blocks_per_sm<16>(finest, src_kind, out);
+        case 4: return level_last_blocks_per_sm<4>(inner, src_kind, out);
+        case 8: return level_last_blocks_per_sm<8>(inner, src_kind, out);
+        case 16: return level_last_blocks_per_sm<16>(inner, src_kind, out);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -11,10 +11,10 @@ cudaError_t launch_level_b(const Pass& p, const PassArgs& a, cudaStream_t st) {
     }
 }
 
-cudaError_t level_occupancy_b(int L, bool finest, int src_kind, int* out) {
+cudaError_t level_occupancy_b(int L, int64_t inner, int src_kind, int* out) {
     switch (L) {
-        case 32: return level_last_blocks_per_sm<32>(finest, src_kind, out);
-        case 64: return level_last_blocks_per_sm<64>(finest, src_kind, out);
+        case 32: return level_last_blocks_per_sm<32>(inner, src_kind, out);
+        case 64: return level_last_blocks_per_sm<64>(inner, src_kind, out);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -42,8 +42,10 @@ __global__ void __launch_bounds__(256) pass_smem(Pass p, PassArgs a) {
     int64_t o = 0, s_first = 0, n_samples = 1, cc = 0;
     if constexpr (MODE == MODE_LAST) {
         cc = b;  // outer == 1
-        s_first = cc * a.tc;
-        n_samples = a.tc;
+        int tb, te;
+        slice_samples(a, tb, te);
+        s_first = cc * a.tc + tb;
+        n_samples = te - tb;
     } else if (rows) {
         o = tile * W;  // first of the CTA's outer lines
         s_first = b;
@@ -131,9 +133,8 @@ __global__ void __launch_bounds__(256) pass_smem(Pass p, PassArgs a) {
     if constexpr (MODE == MODE_LAST) {
         const int64_t i = i0 + w2;
         if (own2 && i < inner) {
-            double* P = a.P + (a.c0 + cc) * a.P_stride + i;
 #pragma unroll
-            for (int k2 = 0; k2 < L2; ++k2) P[(int64_t)(k1 + L1 * k2) * inner] += (double)acc[k2];
+            for (int k2 = 0; k2 < L2; ++k2) fold_last(a, cc, (int64_t)(k1 + L1 * k2) * inner + i, acc[k2]);
         }
     }
 }
@@ -149,7 +150,7 @@ cudaError_t launch_smem_t(const Pass& p, const PassArgs& a, cudaStream_t st) {
     auto k = pass_smem<L1, L2, MODE, SRC>;
     cudaError_t e = smem_limit_once((const void*)k, smem);
     if (e != cudaSuccess) return e;
-    k<<<(unsigned)blocks, threads, smem, st>>>(p, a);
+    k<<<MODE == MODE_LAST ? last_grid(blocks, a) : dim3((unsigned)blocks), threads, smem, st>>>(p, a);
     return cudaGetLastError();
 }
 

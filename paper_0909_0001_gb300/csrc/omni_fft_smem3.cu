@@ -118,8 +118,10 @@ __global__ void __launch_bounds__(s3_threads<MODE>(), 512 / s3_threads<MODE>()) 
         b /= tiles;
         if constexpr (MODE == MODE_LAST) {
             cc = b;  // outer == 1
-            s_first = cc * a.tc;
-            n_samples = a.tc;
+            int tb, te;
+            slice_samples(a, tb, te);
+            s_first = cc * a.tc + tb;
+            n_samples = te - tb;
         } else {
             o0 = b % p.outer;
             s_first = b / p.outer;
@@ -324,7 +326,6 @@ __global__ void __launch_bounds__(s3_threads<MODE>(), 512 / s3_threads<MODE>()) 
     }
     if constexpr (PF) cp_async_wait_all();  // nothing left in flight at exit
     if constexpr (MODE == MODE_LAST) {
-        double* P = a.P + (a.c0 + cc) * a.P_stride;
 #pragma unroll
         for (int u = 0; u < T3; ++u) {
             const int t = tid + u * kS3Threads;
@@ -333,7 +334,7 @@ __global__ void __launch_bounds__(s3_threads<MODE>(), 512 / s3_threads<MODE>()) 
                 if (!line_ok(w)) continue;
 #pragma unroll
                 for (int k3 = 0; k3 < L3; ++k3)
-                    P[(int64_t)(k1 + L1 * k2 + L1 * L2 * k3) * inner + i0 + w] += (double)acc[u][k3];
+                    fold_last(a, cc, (int64_t)(k1 + L1 * k2 + L1 * L2 * k3) * inner + i0 + w, acc[u][k3]);
             }
         }
     }
@@ -362,7 +363,7 @@ cudaError_t launch_s3(const Pass& p, const PassArgs& a, cudaStream_t st) {
     auto k = pass_smem3<L1, L2, L3, W, ROWS, MODE, SRC, PF>;
     cudaError_t e = smem_limit_once((const void*)k, smem);
     if (e != cudaSuccess) return e;
-    k<<<(unsigned)blocks, s3_threads<MODE>(), smem, st>>>(p, a);
+    k<<<MODE == MODE_LAST ? last_grid(blocks, a) : dim3((unsigned)blocks), s3_threads<MODE>(), smem, st>>>(p, a);
     return cudaGetLastError();
 }
 

@@ -87,6 +87,8 @@ struct PassArgs {
     int* err;            // device error word (bounded waits that expired set it to 1)
     int force_expire;    // test hook: make the first bounded wait expire
     double fold_scale;   // FP32 LAST passes: factor on the FP64 fold (0 means 1)
+    int split;           // LAST: slices of the chunk's samples, one grid row each (0 or 1: none)
+    float* part;         // ... each slice's sums [split][S][P_stride], folded by launch_fold_parts
     const float* chan_max;  // per chunk channel: max |re|, |im| of its voltages (KIND_COV5/XSPEC5 with scale_n)
 };
 
@@ -99,6 +101,16 @@ void choose_kind(Pass& p);
 
 // Launch one pass on stream.
 cudaError_t launch_pass(const Pass& p, const PassArgs& a, cudaStream_t stream);
+
+// P[c][e] += fold_scale * sum over the slices of part[slice][c][e], slices in order
+// (after a LAST pass launched with split > 1, on the same stream).
+cudaError_t launch_fold_parts(const PassArgs& a, cudaStream_t stream);
+
+// Columns per CTA of the two-column LAST level pass, 0 where it does not apply (64
+// points; the finest level; odd inner, after unpadded beam axes of odd length).
+constexpr int level_last_columns(int L, int64_t inner = 2) {
+    return L <= 32 && inner > 1 && inner % 2 == 0 ? (L == 16 && inner >= 512 ? 32 : 256 / L) : 0;
+}
 
 // Resident CTAs per SM of the LAST-mode kernel of a KIND_LEVEL pass.
 cudaError_t level_last_occupancy(const Pass& p, int src_kind, int* blocks_per_sm);
