@@ -642,6 +642,9 @@ void choose_chunks(omni_plan* pl) {
     cudaGetLastError();
     int64_t slots = (int64_t)std::max(sms, 1) * std::max(per_sm, 2);
     if (sms <= 0) slots = 304;
+    // 32-point levels: two waves of channels, so that a chunk's FP32 sums stay as short as
+    // with one CTA per SM (256 samples on 4 x 4 tiles on 16 x 16)
+    if (last.kind == KIND_LEVEL && last.L == 32) slots = std::max<int64_t>(slots, 2 * (int64_t)std::max(sms, 152) * per_sm);
     // fill one wave of the last pass: as many channels as the slots hold
     pl->Cc = std::min<int64_t>(pl->C, std::max<int64_t>(1, slots / ctas));
     const int64_t per_sample = std::max<int64_t>(1, pl->fwd_elems) * (int64_t)sizeof(float2);

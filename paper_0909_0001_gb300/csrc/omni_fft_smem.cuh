@@ -19,7 +19,12 @@ namespace omni {
 // Step 2: L2-point FFT along each row k1 gives X[k1 + L1 k2].  Lines along the
 // innermost axis are read and written as contiguous runs: the threads take the
 // points of one line first (j2, or k1, fastest) and the lines second.
-template <int L1, int L2, int MODE, int SRC>
+// WC: the lines per CTA at compile time (256 / L1, 256 threads; the index splits are
+// shifts), or 0 for the fewer lines of a narrow axis.  Each thread's loads are issued
+// together, and a LAST pass of WC lines loads the next sample's inputs into registers
+// while it transforms the current one.  16 arrays-and-channels of 64 x 64 antennas (two
+// 128-point axes, batch of 48): divisions by a run-time W and one load at a time, SMEM_NOW.
+template <int L1, int L2, int MODE, int SRC, int WC>
 __global__ void __launch_bounds__(256) pass_smem(Pass p, PassArgs a) {
     constexpr bool FWD = (MODE == MODE_MID || MODE == MODE_LAST);
     constexpr int L = L1 * L2;
@@ -28,9 +33,10 @@ __global__ void __launch_bounds__(256) pass_smem(Pass p, PassArgs a) {
     constexpr int LOG1 = ilog2(L1), LOG2 = ilog2(L2);
     constexpr int TWS = kTwiddleN / L;
     extern __shared__ float2 sm[];
-    const int W = p.W;
+    const int W = WC ? WC : p.W;
     const int64_t inner = p.inner;
-    const int n = FWD ? L / 2 : L;
+    constexpr int n = FWD ? L / 2 : L;
+    const int NT = WC ? WC * L1 : blockDim.x;
     // lines along the innermost axis: W consecutive outer lines per CTA
     const bool rows = MODE != MODE_LAST && inner == 1;
     const int64_t tiles = rows ? (p.outer + W - 1) / W : (inner + W - 1) / W;
@@ -63,19 +69,56 @@ __global__ void __launch_bounds__(256) pass_smem(Pass p, PassArgs a) {
 #pragma unroll
     for (int k = 0; k < L2; ++k) acc[k] = 0.0f;
 
+    // inputs per thread of one sample (WC), or the loads in flight at a time
+    constexpr int NB = WC ? n / L1 : 8;
+    auto at_e = [&](int e, int& j, int& w) {
+        j = rows ? e % n : e / W;
+        w = rows ? e / n : e % W;
+    };
+    auto load = [&](float2 (&x)[NB], int64_t base, int e0) {
+#pragma unroll
+        for (int r = 0; r < NB; ++r) {
+            const int e = e0 + r * NT;
+            int j, w;
+            at_e(e, j, w);
+            x[r] = (WC || e < n * W) && line_ok(w)
+                       ? ld_src<SRC>(a.src, rows ? base + (int64_t)w * n + j : base + (int64_t)j * inner + w)
+                       : make_float2(0.f, 0.f);
+        }
+    };
+    auto store = [&](const float2 (&x)[NB], int e0) {
+#pragma unroll
+        for (int r = 0; r < NB; ++r) {
+            const int e = e0 + r * NT;
+            int j, w;
+            at_e(e, j, w);
+            if (WC || e < n * W) sm[w * PLANE + (j / L2) * PITCH + (j % L2)] = x[r];
+        }
+    };
+    auto base_of = [&](int64_t s) { return src_base(a, s) + o * (int64_t)n * inner + i0; };
+    constexpr bool AHEAD = WC > 0 && MODE == MODE_LAST && NB <= 8;
+    float2 pre[NB];
+    if constexpr (AHEAD)
+        if (n_samples > 0) load(pre, base_of(s_first), threadIdx.x);
+
     for (int64_t ts = 0; ts < n_samples; ++ts) {
         const int64_t s = s_first + ts;
-        const int64_t base = src_base(a, s) + o * (int64_t)n * inner + i0;
-        // load n inputs of each of the W lines (coalesced over inner, or along each line)
-        for (int e = threadIdx.x; e < n * W; e += blockDim.x) {
-            const int j = rows ? e % n : e / W, w = rows ? e / n : e % W;
-            float2 x = make_float2(0.f, 0.f);
-            if (line_ok(w)) x = ld_src<SRC>(a.src, rows ? base + (int64_t)w * n + j : base + (int64_t)j * inner + w);
-            sm[w * PLANE + (j / L2) * PITCH + (j % L2)] = x;
+        // n inputs of each of the W lines (coalesced over inner, or along each line)
+        if constexpr (AHEAD) {
+            store(pre, threadIdx.x);
+            if (ts + 1 < n_samples) load(pre, base_of(s + 1), threadIdx.x);  // in flight during this sample
+        } else if constexpr (WC > 0) {
+            load(pre, base_of(s), threadIdx.x);
+            store(pre, threadIdx.x);
+        } else {
+            for (int e0 = threadIdx.x; e0 < n * W; e0 += NB * NT) {
+                load(pre, base_of(s), e0);
+                store(pre, e0);
+            }
         }
         __syncthreads();
         // step 1: columns
-        for (int u = threadIdx.x; u < W * L2; u += blockDim.x) {
+        for (int u = threadIdx.x; u < W * L2; u += NT) {
             const int w = rows ? u / L2 : u % W, j2 = rows ? u % L2 : u / W;
             float2* col = sm + w * PLANE + j2;
             float2 v[L1];
@@ -139,6 +182,12 @@ __global__ void __launch_bounds__(256) pass_smem(Pass p, PassArgs a) {
     }
 }
 
+// lines per CTA at compile time: the full tile of 256 threads
+template <int L1, class F>
+cudaError_t with_lines(int W, F&& f) {
+    return W == 256 / L1 ? f(std::integral_constant<int, 256 / L1>{}) : f(std::integral_constant<int, 0>{});
+}
+
 template <int L1, int L2, int MODE, int SRC>
 cudaError_t launch_smem_t(const Pass& p, const PassArgs& a, cudaStream_t st) {
     const bool rows = MODE != MODE_LAST && p.inner == 1;
@@ -147,11 +196,13 @@ cudaError_t launch_smem_t(const Pass& p, const PassArgs& a, cudaStream_t st) {
     if (blocks <= 0) return cudaSuccess;
     const int threads = p.W * L1;
     const size_t smem = (size_t)p.W * (L1 * (L2 + 1) + 1) * sizeof(float2);
-    auto k = pass_smem<L1, L2, MODE, SRC>;
-    cudaError_t e = smem_limit_once((const void*)k, smem);
-    if (e != cudaSuccess) return e;
-    k<<<MODE == MODE_LAST ? last_grid(blocks, a) : dim3((unsigned)blocks), threads, smem, st>>>(p, a);
-    return cudaGetLastError();
+    return with_lines<L1>(p.W, [&](auto W) {
+        auto k = pass_smem<L1, L2, MODE, SRC, decltype(W)::value>;
+        cudaError_t e = smem_limit_once((const void*)k, smem);
+        if (e != cudaSuccess) return e;
+        k<<<MODE == MODE_LAST ? last_grid(blocks, a) : dim3((unsigned)blocks), threads, smem, st>>>(p, a);
+        return cudaGetLastError();
+    });
 }
 
 // Resident CTAs per SM of the LAST-mode kernel of one four-step length.
@@ -160,10 +211,12 @@ cudaError_t smem_last_occupancy_len(const Pass& p, int src_kind, int* blocks_per
     const int threads = p.W * L1;
     const size_t smem = (size_t)p.W * (L1 * (L2 + 1) + 1) * sizeof(float2);
     return dispatch_src<MODE_LAST>(src_kind, [&](auto S) {
-        auto k = pass_smem<L1, L2, MODE_LAST, decltype(S)::value>;
-        cudaError_t e = smem_limit_once((const void*)k, smem);
-        if (e != cudaSuccess) return e;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem);
+        return with_lines<L1>(p.W, [&](auto W) {
+            auto k = pass_smem<L1, L2, MODE_LAST, decltype(S)::value, decltype(W)::value>;
+            cudaError_t e = smem_limit_once((const void*)k, smem);
+            if (e != cudaSuccess) return e;
+            return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, threads, smem);
+        });
     });
 }
 
