@@ -9,7 +9,7 @@
 // The real frame is packed as F complex points z(m) = u(2m) + i u(2m+1), run
 // through an F-point FFT and unpacked to the real spectrum, in one pass over the
 // samples: fengine64 (F = 64 and 16-byte sample rows), fengine_multi (other F >= 16),
-// fengine_fused (F < 16).  int8 outputs round half to even and clip to +-127.
+// fengine_fused (F < 16, and few samples of up to 256 channels).  int8 outputs round half to even and clip to +-127.
 #include "omni_fft_common.cuh"
 #include "omni.h"
 
@@ -45,7 +45,7 @@ constexpr int kFuseAnt = 16;     // antennas per CTA: 32-byte int8 output rows
 constexpr int kFusePoints = 4096;  // complex points in shared memory (32 KB)
 static_assert(kFuseAnt == 16 && kFusePoints / kFuseAnt == 256, "fused index shifts assume 16 x 256 points");
 
-// Fused F-engine for small F: CTA = (16 consecutive antennas, FR frames),
+// Fused F-engine for small F or few samples: CTA = (16 consecutive antennas, FR frames),
 // FR = 256 / F; polyphase, FFT, unpacking, calibration and quantisation in
 // shared memory, each output row (channel f, frame t) written as the 16
 // antennas' values together, so no intermediate spectrum goes through HBM.
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kFThreads) fengine_fused(const int8_t* __restr
 // 72: the half-warps of every step touch 16 different bank pairs.
 // 16384 antennas, 4 taps, 1024 frames, int8 out: 6.33 -> 3.59 ms.
 constexpr int kF64Ant = 32;
-constexpr int kF64Frames = 16;
+constexpr int kF64Frames = 16;  // most frames per CTA; fewer (even) while the GPU is not filled
 constexpr int kF64MaxTaps = 8;
 constexpr int kF64Row = 36;  // char2 per staged row (72 bytes: conflict-free 2-byte stores and 8-byte loads)
 
@@ -194,7 +194,7 @@ template <bool I8, bool GAINS>
 __global__ void __launch_bounds__(256, 2) fengine64(const int8_t* __restrict__ raw, int64_t N, int64_t S, int P,
                                                     const float* __restrict__ w, int64_t T,
                                                     const float2* __restrict__ gains, float scale,
-                                                    void* __restrict__ out) {
+                                                    void* __restrict__ out, int frames) {
     __shared__ float2 zs[8][4 * 72];                                 // per warp: 4 transforms
     __shared__ __align__(16) char2 yq[2][2][I8 ? 64 : 1][kF64Row];   // [pair parity][frame][channel][antenna]
     __shared__ __align__(16) float wsm[kF64MaxTaps * 128];           // [tap][quarter][lane][4]: w(16 lane + 4 quarter ..)
@@ -202,8 +202,8 @@ __global__ void __launch_bounds__(256, 2) fengine64(const int8_t* __restrict__ r
     const int tr = lane >> 3, l = lane & 7;
     for (int i = tid; i < P * 128; i += 256)
         wsm[i] = w ? w[(i & ~127) + ((i >> 2) & 7) * 16 + ((i >> 5) & 3) * 4 + (i & 3)] : 1.f;
-    const int64_t tchunks = (T + kF64Frames - 1) / kF64Frames;
-    const int64_t a0 = (blockIdx.x / tchunks) * kF64Ant, t0 = (blockIdx.x % tchunks) * kF64Frames;
+    const int64_t tchunks = (T + frames - 1) / frames;
+    const int64_t a0 = (blockIdx.x / tchunks) * kF64Ant, t0 = (blockIdx.x % tchunks) * frames;
     const int al = 4 * warp + tr;  // antenna within the CTA
     const int64_t a = a0 + al;
     const int64_t last = a < N ? T + P - 1 : 0;  // frames of this antenna that exist
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(256, 2) fengine64(const int8_t* __restrict__ r
         for (int b = 0; b < 16; ++b) d[b] = (float)(int8_t)(q[b >> 2] >> (8 * (b & 3)));
     };
     uint4 f0 = fetch(t0), f1 = fetch(t0 + 1);
-    for (int64_t t = t0; t < t0 + kF64Frames && t < T; t += 2) {
+    for (int64_t t = t0; t < t0 + frames && t < T; t += 2) {
         // polyphase sums of samples 16 l .. 16 l + 15 of frames t and t + 1:
         // z(8 l + q) = u(16 l + 2q) + i u(16 l + 2q + 1)
         float u0[16], u1[16];
@@ -682,13 +682,21 @@ cudaError_t launch_fengine(const int8_t* raw, int64_t N, int64_t S, int32_t F, i
     }
     const bool vec = F >= 8 && S % 16 == 0 && (uintptr_t)raw % 16 == 0 && (uintptr_t)window % 16 == 0;
     if (F == 64 && vec && P <= kF64MaxTaps) {
-        const unsigned c64 = (unsigned)(((N + kF64Ant - 1) / kF64Ant) * ((T + kF64Frames - 1) / kF64Frames));
+        int frames = kF64Frames;
+        const int64_t groups = (N + kF64Ant - 1) / kF64Ant;
+        while (frames > 2 && groups * ((T + frames - 1) / frames) < 152) frames /= 2;
+        const unsigned c64 = (unsigned)(groups * ((T + frames - 1) / frames));
         auto k = out_i8 ? (gains ? fengine64<true, true> : fengine64<true, false>)
                         : (gains ? fengine64<false, true> : fengine64<false, false>);
-        k<<<c64, 256, 0, st>>>(raw, N, S, P, window, T, gains, scale, out);
+        k<<<c64, 256, 0, st>>>(raw, N, S, P, window, T, gains, scale, out, frames);
         return cudaGetLastError();
     }
-    switch (logF) {
+    // up to 256 channels the CTA of the pass above takes 4096 / F antennas, twice what the
+    // radix-2 pass does in points: with fewer antennas, or too few points for one CTA per SM,
+    // the smaller CTAs win (8 antennas, 16 channels, 4 taps, 2048 frames: 14 against 30 us; 64
+    // antennas, 256 channels, 16 frames: 21 against 27)
+    const bool small = F <= 256 && (N < 4096 / F || N * T * F < (int64_t)152 * 8192);
+    switch (small ? 0 : logF) {
 #define OMNI_MULTI(n) \
     case n: return launch_multi<n>(raw, N, S, P, window, T, gains, scale, out, out_i8, st)
         OMNI_MULTI(4);
@@ -701,7 +709,7 @@ cudaError_t launch_fengine(const int8_t* raw, int64_t N, int64_t S, int32_t F, i
         OMNI_MULTI(11);
         OMNI_MULTI(12);
 #undef OMNI_MULTI
-        default: break;  // F < 16
+        default: break;  // F < 16, or small
     }
     const unsigned ctas = (unsigned)fengine_ctas(N, T, F);
     if (out_i8 && vec)

@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(256) pass_reg(Pass p, PassArgs a) {
 // per line as above, but its points are contiguous in memory, so that a thread reading
 // and writing its own line touches 32 lines of memory per warp access (2.3 TB/s, 16-byte
 // outputs).  The CTA's lines go through shared memory and memory is read and written in
-// runs: one 16 x 16 on 8 x 8 hierarchy, 64 channels, last inverse pass: 149 -> ROWS_NOW us.
+// runs: one 16 x 16 on 8 x 8 hierarchy, 64 channels, last inverse pass: 149 -> 117 us.
 template <int L, int MODE, int SRC>
 __global__ void __launch_bounds__(128) pass_reg_rows(Pass p, PassArgs a) {
     constexpr bool FWD = MODE == MODE_MID;

@@ -22,8 +22,9 @@ namespace omni {
 // WC: the lines per CTA at compile time (256 / L1, 256 threads; the index splits are
 // shifts), or 0 for the fewer lines of a narrow axis.  Each thread's loads are issued
 // together, and a LAST pass of WC lines loads the next sample's inputs into registers
-// while it transforms the current one.  16 arrays-and-channels of 64 x 64 antennas (two
-// 128-point axes, batch of 48): divisions by a run-time W and one load at a time, SMEM_NOW.
+// while it transforms the current one.  A batch's 64 x 64 arrays (two
+// 128-point axes, 16 channels x 512 samples): divisions by a run-time W and one load at a time, 2.72 +
+// 4.07 ms, now 1.94 + 2.03.
 template <int L1, int L2, int MODE, int SRC, int WC>
 __global__ void __launch_bounds__(256) pass_smem(Pass p, PassArgs a) {
     constexpr bool FWD = (MODE == MODE_MID || MODE == MODE_LAST);

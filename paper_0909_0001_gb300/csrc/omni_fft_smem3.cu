@@ -11,44 +11,37 @@
 // (the factorisation of w_L^(j k) into the three DFTs and two twiddle stages).
 // The inverse passes use the same transform (the inverse runs as a forward FFT)
 // on all L inputs and keep the lag slots, the last one conjugated and scaled.
-// A CTA transforms W lines held in shared memory as [j1][j2][j3] with a row pitch
-// L3 + 1, a j1 pitch = 8 and a line pitch = 16 / W (mod 16) float2, so that each
-// step's half-warps touch 16 different bank pairs; each thread reads one twiddle w^j from
-// a shared-memory table (LAST: through L1) and forms the powers it needs in
-// registers.  LAST runs two 256-thread CTAs per SM and, reading the scratch
-// buffer, copies the next sample's inputs asynchronously (cp.async) into a staging
-// buffer while the current sample runs steps 2 and 3.  Lines
-// are W consecutive inner indices (strided axes), or, for an axis that is
-// innermost in memory, W consecutive outer lines read and written contiguously.
-// MID and the inverse passes write through shared memory in natural order; LAST keeps
-// |X|^2 of the chunk's samples in registers and folds them into the FP64
-// accumulator once.  The forward inputs j >= L/2 are zero (padding): step 1
-// never reads them.
+// A 256-thread CTA, two per SM, transforms W lines in pairs: each shared-memory element
+// is one point of two lines (re, re, im, im), so that a point is one 16-byte access, the
+// butterflies run on both lines per f32x2 instruction and the twiddle powers are formed
+// once for both.  A line pair is held as [j1][j2][j3] with a row pitch L3 + 1, so that
+// each step's quarter-warps touch 8 different 16-byte banks (j1 pitch
+// 1, pair pitch 4, mod 8); each thread reads one
+// twiddle w^j through L1 and forms the powers it needs in registers.  LAST, reading the
+// scratch buffer, copies the next sample's inputs asynchronously (cp.async) into a staging
+// buffer while the current sample runs steps 2 and 3.  Lines are W consecutive inner
+// indices (strided axes), or, for an axis that is innermost in memory, W consecutive
+// outer lines read and written contiguously: step 1 takes its inputs from memory and step 3,
+// whose bins are consecutive across a warp, writes its outputs there.  LAST keeps |X|^2 of the chunk's samples in registers and
+// folds them into the FP64 accumulator once.  The forward inputs j >= L/2 are zero
+// (padding): step 1 never reads them.
+// What bounds it is shared memory (four 8-byte passes per point and line) and FP32.  1024 x 1024 antennas (2048-point axes),
+// 64 samples, line by line at 512 (LAST 256) threads against pairs, serial:
+// MID 0.48 -> 0.30 ms (5.4 TB/s), LAST 0.65 -> 0.52 ms (inputs and outputs through shared memory
+// too, in pairs: 0.42 and 0.63).
 #include "omni_fft_common.cuh"
 
 namespace omni {
 namespace {
 
-// threads per CTA: 512, or 256 for LAST (whose 32 FP32 |X|^2 sums per thread and
-// ~120 registers would otherwise leave one CTA per SM and no overlap of one CTA's
-// loads with another's transforms)
-template <int MODE>
-__host__ __device__ constexpr int s3_threads() { return MODE == MODE_LAST ? 256 : 512; }
+constexpr int kS3Threads = 256;
 
-template <int L1, int L2, int L3, int W>
+template <int L1, int L2, int L3>
 struct S3Geom {
     static constexpr int L = L1 * L2 * L3, M = L2 * L3;
-    static constexpr int P2 = L3 + 1;
-    static constexpr int P1 = L2 * P2 + ((8 - (L2 * P2) % 16 + 16) % 16);
-    // lines 16 / W float2 apart mod 16: the W lines x 16 / W consecutive inputs of a
-    // half-warp's strided load land in 16 different bank pairs
-    static constexpr int PG = (16 / W) % 16;
-    static constexpr int PLANE = L1 * P1 + ((PG - (L1 * P1) % 16 + 16) % 16);
-    static_assert(P1 % 16 == 8 && PLANE % 16 == PG, "pitches");
-    static_assert(PLANE >= L + L / 16, "the natural-order output fits the plane");
+    static constexpr int P2 = L3 + 1, P1 = L2 * P2 + 1, PLANE = L1 * P1 + (12 - L1 * P1 % 8) % 8;
+    static_assert(P2 % 8 == 1 && P1 % 8 == 1 && PLANE % 8 == 4, "16-byte points on different banks");
 };
-
-__device__ __forceinline__ int out_at(int k) { return k + (k >> 4); }  // natural order, 1 pad per 16
 
 // 16-byte asynchronous copy global -> shared (zero-filled when !valid; src must
 // still be a valid address)
@@ -79,31 +72,39 @@ struct Pow16 {
     }
 };
 
+// one point of two lines, as it lies in shared memory and in registers
+__device__ __forceinline__ void get2(const float4* p, f2x& x, f2x& y) {
+    const float4 q = *p;
+    x = pack2(q.x, q.y);
+    y = pack2(q.z, q.w);
+}
+__device__ __forceinline__ void put2(float4* p, f2x x, f2x y) {
+    const float2 a = unpack2(x), b = unpack2(y);
+    *p = make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void cmul2(f2x& x, f2x& y, float2 w) {
+    const f2x c = dup2(w.x), t = x;
+    x = fma2(t, c, mul2(y, dup2(-w.y)));
+    y = fma2(t, dup2(w.y), mul2(y, c));
+}
+
 // PF (LAST from the float2 scratch buffer, 16-byte aligned rows): the next
 // sample's W x L/2 inputs are copied asynchronously into a staging buffer
 // [j][W] while the current sample runs steps 2 and 3, and step 1 reads them there.
 template <int L1, int L2, int L3, int W, bool ROWS, int MODE, int SRC, bool PF>
-__global__ void __launch_bounds__(s3_threads<MODE>(), 512 / s3_threads<MODE>()) pass_smem3(Pass p, PassArgs a) {
-    constexpr int kS3Threads = s3_threads<MODE>();
-    using G = S3Geom<L1, L2, L3, W>;
-    static_assert(!PF || (MODE == MODE_LAST && SRC == SRC_BUF && !ROWS && W % 2 == 0), "prefetch form");
+__global__ void __launch_bounds__(kS3Threads, 2) pass_smem3(Pass p, PassArgs a) {
+    using G = S3Geom<L1, L2, L3>;
+    static_assert(!PF || (MODE == MODE_LAST && SRC == SRC_BUF && !ROWS), "prefetch form");
     constexpr int L = G::L, M = G::M, P1 = G::P1, P2 = G::P2, PLANE = G::PLANE;
     constexpr bool FWD = MODE == MODE_MID || MODE == MODE_LAST;  // forward: inputs j >= L/2 are zero
-    constexpr int LOG1 = ilog2(L1), LOG2 = ilog2(L2), LOG3 = ilog2(L3);
-    constexpr int T1 = (W * M + kS3Threads - 1) / kS3Threads;       // step-1 tasks per thread
-    constexpr int T2 = (W * L1 * L3 + kS3Threads - 1) / kS3Threads;  // step 2
-    constexpr int T3 = (W * L1 * L2 + kS3Threads - 1) / kS3Threads;  // step 3
-    // LAST reads its twiddles through L1 (its shared memory holds the lines and,
-    // with PF, the staging buffer of two CTAs per SM); the others keep a table
-    constexpr bool TWG = MODE == MODE_LAST;
-    extern __shared__ float2 sm[];
-    float2* tw = sm;                    // [L]: w_L^m (not TWG)
-    float2* lines = sm + (TWG ? 0 : L); // [W][PLANE]
-    float2* stage = lines + W * PLANE;  // PF: [L/2][W]
+    constexpr int LOG1 = ilog2(L1), LOG2 = ilog2(L2), LOG3 = ilog2(L3), H = W / 2;
+    static_assert(W % 2 == 0 && H * M == kS3Threads && H * L1 * L3 == kS3Threads, "one task per thread, steps 1 and 2");
+    constexpr int T3 = H * L1 * L2 / kS3Threads;  // step-3 tasks per thread
+    extern __shared__ float4 sm4[];
+    float4* lines = sm4;                                            // [H][PLANE]
+    float2* stage = reinterpret_cast<float2*>(lines + H * PLANE);   // PF: [L/2][W]
     const int tid = threadIdx.x;
-    if constexpr (!TWG)
-        for (int m = tid; m < L; m += kS3Threads) tw[m] = g_tw4096[m * (kTwiddleN / L)];
-    auto twv = [&](int m) { return TWG ? __ldg(&g_tw4096[m * (kTwiddleN / L)]) : tw[m]; };
+    auto twv = [&](int m) { return __ldg(&g_tw4096[m * (kTwiddleN / L)]); };
 
     const int n = p.n;  // inputs per line (<= L / 2 forward, <= L inverse)
     const int64_t inner = p.inner;
@@ -130,21 +131,21 @@ __global__ void __launch_bounds__(s3_threads<MODE>(), 512 / s3_threads<MODE>()) 
     // the lines this CTA has (the last tile may be short)
     auto line_ok = [&](int w) { return ROWS ? o0 + w < p.outer : i0 + w < inner; };
 
-    float acc[T3][L3];
+    f2x acc[MODE == MODE_LAST ? T3 : 1][L3];
 #pragma unroll
-    for (int u = 0; u < T3; ++u)
+    for (int u = 0; u < (MODE == MODE_LAST ? T3 : 1); ++u)
 #pragma unroll
-        for (int k = 0; k < L3; ++k) acc[u][k] = 0.f;
+        for (int k = 0; k < L3; ++k) acc[u][k] = dup2(0.f);
 
     // PF: one sample's inputs, 16 bytes (two lines) per copy; rows j >= n and lines
     // past the axis are zero-filled
     auto prefetch = [&](int64_t s) {
         const float2* row0 = reinterpret_cast<const float2*>(a.src) + s * a.src_stride + i0;
-        constexpr int CH = W / 2, NC = (L / 2) * CH / kS3Threads;
-        static_assert(NC * kS3Threads == (L / 2) * CH, "copies per thread");
+        constexpr int NC = (L / 2) * H / kS3Threads;
+        static_assert(NC * kS3Threads == (L / 2) * H, "copies per thread");
 #pragma unroll
         for (int r = 0; r < NC; ++r) {
-            const int c = tid + r * kS3Threads, j = c / CH, h = c % CH;
+            const int c = tid + r * kS3Threads, j = c / H, h = c % H;
             const bool ok = j < n && i0 + 2 * h < inner;
             cp_async16(stage + j * W + 2 * h, ok ? row0 + (int64_t)j * inner + 2 * h : row0, ok);
         }
@@ -156,195 +157,128 @@ __global__ void __launch_bounds__(s3_threads<MODE>(), 512 / s3_threads<MODE>()) 
     for (int64_t ts = 0; ts < n_samples; ++ts) {
         const int64_t s = s_first + ts;
         const int64_t base = src_base(a, s);
-        // load: contiguous runs along the line (ROWS) or W inner indices per input,
-        // each thread's loads issued together before its shared-memory stores
-        auto at_j = [&](int w, int j) { return w * PLANE + (j / M) * P1 + ((j / L3) % L2) * P2 + (j % L3); };
         if constexpr (PF) {
-            cp_async_wait_all();  // this sample's staging copies (the barrier below publishes them)
-        } else if constexpr (ROWS) {
-            constexpr int NR = (FWD ? L / 2 : L) / kS3Threads;  // loads per line and thread
-            float2 x[W][NR];
+            cp_async_wait_all();  // this sample's staging copies
+            __syncthreads();      // ... everyone's, and the lines are free
+        }
+        // step 1: j' = j3 + L3 j2 fastest across the threads (strided axes: the line pairs), inputs
+        // straight from the staging buffer or from memory, all of a thread's loads together
+        {
+            const int h = ROWS ? tid / M : tid % H, jp = ROWS ? tid - h * M : tid / H, j2 = jp / L3, j3 = jp - j2 * L3;
+            float4* col = lines + h * PLANE + j2 * P2 + j3;
+            f2x x[L1], y[L1];
+            constexpr int NIN = FWD ? L1 / 2 : L1;
+            if constexpr (PF) {
 #pragma unroll
-            for (int w = 0; w < W; ++w)
-#pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    const int j = tid + r * kS3Threads;
-                    x[w][r] = (j < n && line_ok(w)) ? ld_src<SRC>(a.src, base + (o0 + w) * (int64_t)n + j)
-                                                    : make_float2(0.f, 0.f);
+                for (int j1 = 0; j1 < NIN; ++j1) {
+                    const float4 q = *reinterpret_cast<const float4*>(stage + (jp + M * j1) * W + 2 * h);
+                    x[j1] = pack2(q.x, q.z);
+                    y[j1] = pack2(q.y, q.w);
                 }
+            } else {
+                const bool ok0 = line_ok(2 * h), ok1 = line_ok(2 * h + 1);
+                const int64_t first = ROWS ? base + (o0 + 2 * h) * (int64_t)n : base + o0 * (int64_t)n * inner + i0 + 2 * h;
+                const int64_t next = ROWS ? n : 1, step = ROWS ? 1 : inner;  // to the second line; to the next input
 #pragma unroll
-            for (int w = 0; w < W; ++w)
-#pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    const int j = tid + r * kS3Threads;
-                    if (j < n) lines[at_j(w, j)] = x[w][r];
-                }
-        } else {
-            constexpr int NB = 16;  // loads in flight per thread
-            const int n_in = W * n;
-            const int64_t col = base + o0 * (int64_t)n * inner + i0;
-            for (int e0 = 0; e0 < n_in; e0 += NB * kS3Threads) {
-                float2 x[NB];
-#pragma unroll
-                for (int r = 0; r < NB; ++r) {
-                    const int e = e0 + tid + r * kS3Threads, j = e / W, w = e % W;
-                    x[r] = (e < n_in && line_ok(w)) ? ld_src<SRC>(a.src, col + (int64_t)j * inner + w)
-                                                    : make_float2(0.f, 0.f);
-                }
-#pragma unroll
-                for (int r = 0; r < NB; ++r) {
-                    const int e = e0 + tid + r * kS3Threads;
-                    if (e < n_in) lines[at_j(e % W, e / W)] = x[r];
+                for (int j1 = 0; j1 < NIN; ++j1) {
+                    const int j = jp + M * j1;
+                    const float2 zero = make_float2(0.f, 0.f);
+                    const float2 u = j < n && ok0 ? ld_src<SRC>(a.src, first + j * step) : zero;
+                    const float2 v = j < n && ok1 ? ld_src<SRC>(a.src, first + next + j * step) : zero;
+                    x[j1] = pack2(u.x, v.x);
+                    y[j1] = pack2(u.y, v.y);
                 }
             }
-        }
-        __syncthreads();
-        // step 1: j' = j3 + L3 j2 fastest across the threads
 #pragma unroll
-        for (int u = 0; u < T1; ++u) {
-            const int t = tid + u * kS3Threads;
-            if (t < W * M) {
-                // PF: the W lines fastest (the half-warp reads 16 consecutive staged inputs)
-                const int w = PF ? t % W : t / M, jp = PF ? t / W : t - w * M, j2 = jp / L3, j3 = jp - j2 * L3;
-                float2* col = lines + w * PLANE + j2 * P2 + j3;
-                float2 v[L1];
+            for (int j1 = NIN; j1 < L1; ++j1) x[j1] = y[j1] = dup2(0.f);
+            fft_dif2<L1, FWD>(x, y);
+            const Pow16 pw(twv(jp));  // w_L^(j' k1)
 #pragma unroll
-                for (int j1 = 0; j1 < L1; ++j1) {
-                    if constexpr (PF)
-                        v[j1] = j1 < L1 / 2 ? stage[(jp + M * j1) * W + w] : make_float2(0.f, 0.f);
-                    else
-                        v[j1] = (!FWD || j1 < L1 / 2) ? col[j1 * P1] : make_float2(0.f, 0.f);
-                }
-                fft_dif<L1, FWD>(v);
-                const Pow16 pw(twv(jp));  // w_L^(j' k1)
-#pragma unroll
-                for (int k1 = 0; k1 < L1; ++k1) {
-                    float2 y = v[brev(k1, LOG1)];
-                    if (k1) y = cmul(y, pw(k1));
-                    col[k1 * P1] = y;
-                }
+            for (int k1 = 0; k1 < L1; ++k1) {
+                f2x &vx = x[brev(k1, LOG1)], &vy = y[brev(k1, LOG1)];
+                if (k1) cmul2(vx, vy, pw(k1));
+                put2(col + k1 * P1, vx, vy);
             }
         }
         __syncthreads();
         if constexpr (PF)
             if (ts + 1 < n_samples) prefetch(s + 1);  // the staging buffer is free until the next step 1
         // step 2: (k1, j3), j3 fastest
+        {
+            const int j3 = tid % L3, k1 = (tid / L3) % L1, h = tid / (L3 * L1);
+            float4* row = lines + h * PLANE + k1 * P1 + j3;
+            f2x x[L2], y[L2];
 #pragma unroll
-        for (int u = 0; u < T2; ++u) {
-            const int t = tid + u * kS3Threads;
-            if (t < W * L1 * L3) {
-                const int j3 = t % L3, k1 = (t / L3) % L1, w = t / (L3 * L1);
-                float2* row = lines + w * PLANE + k1 * P1 + j3;
-                float2 v[L2];
+            for (int j2 = 0; j2 < L2; ++j2) get2(row + j2 * P2, x[j2], y[j2]);
+            fft_dif2<L2, false>(x, y);
+            const Pow16 pw(twv(L1 * j3));  // w_M^(j3 k2) = w_L^(L1 j3 k2)
 #pragma unroll
-                for (int j2 = 0; j2 < L2; ++j2) v[j2] = row[j2 * P2];
-                fft_dif<L2, false>(v);
-                const Pow16 pw(twv(L1 * j3));  // w_M^(j3 k2) = w_L^(L1 j3 k2)
-#pragma unroll
-                for (int k2 = 0; k2 < L2; ++k2) {
-                    float2 y = v[brev(k2, LOG2)];
-                    if (k2) y = cmul(y, pw(k2));
-                    row[k2 * P2] = y;
-                }
+            for (int k2 = 0; k2 < L2; ++k2) {
+                f2x &vx = x[brev(k2, LOG2)], &vy = y[brev(k2, LOG2)];
+                if (k2) cmul2(vx, vy, pw(k2));
+                put2(row + k2 * P2, vx, vy);
             }
         }
         __syncthreads();
-        // step 3: (k1, k2), k2 fastest; X[k1 + L1 k2 + L1 L2 k3]
-        float2 out[T3][L3];
+        // step 3: (k1, k2), k1 fastest: X[k1 + L1 k2 + L1 L2 k3], so that a warp's outputs of one
+        // k3 are consecutive bins and go straight out
 #pragma unroll
         for (int u = 0; u < T3; ++u) {
             const int t = tid + u * kS3Threads;
-            if (t < W * L1 * L2) {
-                const int k2 = t % L2, k1 = (t / L2) % L1, w = t / (L2 * L1);
-                const float2* r = lines + w * PLANE + k1 * P1 + k2 * P2;
-                float2 v[L3];
+            const int h = ROWS ? t / (L1 * L2) : t % H, k12 = ROWS ? t % (L1 * L2) : t / H, k1 = k12 % L1, k2 = k12 / L1;
+            const float4* r = lines + h * PLANE + k1 * P1 + k2 * P2;
+            f2x x[L3], y[L3];
 #pragma unroll
-                for (int j3 = 0; j3 < L3; ++j3) v[j3] = r[j3];
-                fft_dif<L3, false>(v);
+            for (int j3 = 0; j3 < L3; ++j3) get2(r + j3, x[j3], y[j3]);
+            fft_dif2<L3, false>(x, y);
+            const bool ok0 = line_ok(2 * h), ok1 = line_ok(2 * h + 1);
 #pragma unroll
-                for (int k3 = 0; k3 < L3; ++k3) {
-                    out[u][k3] = v[brev(k3, LOG3)];
-                    if constexpr (MODE == MODE_LAST) acc[u][k3] += cnorm(out[u][k3]);
+            for (int k3 = 0; k3 < L3; ++k3) {
+                const f2x vx = x[brev(k3, LOG3)], vy = y[brev(k3, LOG3)];
+                if constexpr (MODE == MODE_LAST) {
+                    acc[u][k3] = add2(acc[u][k3], fma2(vx, vx, mul2(vy, vy)));
+                } else {
+                    // forward: slot k; inverse: the slot of lag k or k - L, if it is kept (the last pass
+                    // conjugates and scales: the inverse runs as a forward FFT)
+                    const int k = k12 + L1 * L2 * k3, Q = FWD ? L : p.q_out;
+                    const int q = FWD ? k : (k < L - p.q_shift ? k : k - L) + p.q_shift;
+                    if (!FWD && q >= Q) continue;
+                    const float2 re = unpack2(vx), im = unpack2(vy);
+                    const int64_t at = ROWS ? (o0 + 2 * h) * (int64_t)Q + q : (o0 * Q + q) * inner + i0 + 2 * h;
+                    const int64_t second = at + (ROWS ? Q : 1);
+                    if constexpr (MODE == MODE_INV_LAST) {
+                        double2* V = a.V + (a.c0 + s) * a.V_stride;
+                        if (ok0) V[at] = make_double2((double)re.x * a.scale, -(double)im.x * a.scale);
+                        if (ok1) V[second] = make_double2((double)re.y * a.scale, -(double)im.y * a.scale);
+                    } else {
+                        float2* d = a.dst + s * a.dst_stride;
+                        if (ok0) d[at] = make_float2(re.x, im.x);
+                        if (ok1) d[second] = make_float2(re.y, im.y);
+                    }
                 }
             }
         }
-        if constexpr (MODE != MODE_LAST) {
-            // the spectrum in natural order through shared memory, then contiguous stores
-            __syncthreads();
-#pragma unroll
-            for (int u = 0; u < T3; ++u) {
-                const int t = tid + u * kS3Threads;
-                if (t < W * L1 * L2) {
-                    const int k2 = t % L2, k1 = (t / L2) % L1, w = t / (L2 * L1);
-#pragma unroll
-                    for (int k3 = 0; k3 < L3; ++k3)
-                        lines[w * PLANE + out_at(k1 + L1 * k2 + L1 * L2 * k3)] = out[u][k3];
-                }
-            }
-            __syncthreads();
-            if constexpr (!FWD) {
-                // inverse: the kept lags, slot q = bin (q - q_shift) mod L; the last
-                // pass conjugates and scales (the inverse runs as a forward FFT)
-                const int Q = p.q_out;
-                for (int e = tid; e < W * Q; e += kS3Threads) {
-                    int w, q;
-                    if constexpr (ROWS) {
-                        w = e / Q;
-                        q = e - w * Q;
-                    } else {
-                        q = e / W;
-                        w = e - q * W;
-                    }
-                    if (!line_ok(w)) continue;
-                    const float2 x = lines[w * PLANE + out_at(inv_bin(q, p.q_shift, L))];
-                    const int64_t o = ROWS ? o0 + w : o0, i = ROWS ? 0 : i0 + w;
-                    const int64_t at = (o * Q + q) * inner + i;
-                    if constexpr (MODE == MODE_INV_MID)
-                        a.dst[s * a.dst_stride + at] = x;
-                    else
-                        a.V[(a.c0 + s) * a.V_stride + at] = make_double2((double)x.x * a.scale, -(double)x.y * a.scale);
-                }
-            } else {
-                float2* d = a.dst + s * a.dst_stride;
-                for (int e = tid; e < W * L; e += kS3Threads) {
-                    int w, k;
-                    if constexpr (ROWS) {
-                        w = e / L;
-                        k = e - w * L;
-                    } else {
-                        k = e / W;
-                        w = e - k * W;
-                    }
-                    if (!line_ok(w)) continue;
-                    const float2 x = lines[w * PLANE + out_at(k)];
-                    if constexpr (ROWS) d[(o0 + w) * (int64_t)L + k] = x;
-                    else d[o0 * (int64_t)L * inner + (int64_t)k * inner + i0 + w] = x;
-                }
-            }
-        }
-        __syncthreads();
+        if (!PF && ts + 1 < n_samples) __syncthreads();  // the lines are free (PF: at the next sample's barrier)
     }
     if constexpr (PF) cp_async_wait_all();  // nothing left in flight at exit
     if constexpr (MODE == MODE_LAST) {
 #pragma unroll
         for (int u = 0; u < T3; ++u) {
-            const int t = tid + u * kS3Threads;
-            if (t < W * L1 * L2) {
-                const int k2 = t % L2, k1 = (t / L2) % L1, w = t / (L2 * L1);
-                if (!line_ok(w)) continue;
+            const int t = tid + u * kS3Threads, h = t % H, k12 = t / H;
 #pragma unroll
-                for (int k3 = 0; k3 < L3; ++k3)
-                    fold_last(a, cc, (int64_t)(k1 + L1 * k2 + L1 * L2 * k3) * inner + i0 + w, acc[u][k3]);
+            for (int k3 = 0; k3 < L3; ++k3) {
+                const float2 v = unpack2(acc[u][k3]);
+                const int64_t at = (int64_t)(k12 + L1 * L2 * k3) * inner + i0 + 2 * h;
+                if (line_ok(2 * h)) fold_last(a, cc, at, v.x);
+                if (line_ok(2 * h + 1)) fold_last(a, cc, at + 1, v.y);
             }
         }
     }
 }
 
-template <int L1, int L2, int L3, int W, int MODE, bool PF>
+template <int L1, int L2, int L3, int W, bool PF>
 constexpr size_t s3_smem() {
-    constexpr int L = L1 * L2 * L3;
-    return sizeof(float2) * ((MODE == MODE_LAST ? 0 : (size_t)L) + (size_t)W * S3Geom<L1, L2, L3, W>::PLANE +
-                             (PF ? (size_t)W * (L / 2) : 0));
+    return sizeof(float4) * (W / 2) * S3Geom<L1, L2, L3>::PLANE + (PF ? sizeof(float2) * W * (L1 * L2 * L3 / 2) : 0);
 }
 
 // the prefetch form: LAST from the scratch buffer with 16-byte aligned input rows
@@ -359,25 +293,24 @@ cudaError_t launch_s3(const Pass& p, const PassArgs& a, cudaStream_t st) {
     if (ROWS) blocks = a.S * ((p.outer + W - 1) / W);
     else blocks = (MODE == MODE_LAST ? a.S : a.S * p.outer) * ((p.inner + W - 1) / W);
     if (blocks <= 0) return cudaSuccess;
-    constexpr size_t smem = s3_smem<L1, L2, L3, W, MODE, PF>();
+    constexpr size_t smem = s3_smem<L1, L2, L3, W, PF>();
     auto k = pass_smem3<L1, L2, L3, W, ROWS, MODE, SRC, PF>;
     cudaError_t e = smem_limit_once((const void*)k, smem);
     if (e != cudaSuccess) return e;
-    k<<<MODE == MODE_LAST ? last_grid(blocks, a) : dim3((unsigned)blocks), s3_threads<MODE>(), smem, st>>>(p, a);
+    k<<<MODE == MODE_LAST ? last_grid(blocks, a) : dim3((unsigned)blocks), kS3Threads, smem, st>>>(p, a);
     return cudaGetLastError();
 }
 
-// one length: lines along a strided axis (W = WC; WL for LAST) or along the innermost axis (W = WR)
-template <int L1, int L2, int L3, int WC, int WR, int WL>
+// one length: W lines along a strided axis or along the innermost axis
+template <int L1, int L2, int L3, int W>
 cudaError_t launch_s3_len(const Pass& p, const PassArgs& a, cudaStream_t st) {
     const bool fwd = p.mode == MODE_MID || p.mode == MODE_LAST;
-    if (p.n > (fwd ? L1 * L2 * L3 / 2 : L1 * L2 * L3)) return cudaErrorInvalidValue;
+    if (p.n > (fwd ? L1 * L2 * L3 / 2 : L1 * L2 * L3) || p.W != W) return cudaErrorInvalidValue;
     const bool rows = p.mode != MODE_LAST && p.inner == 1;
-    if (p.W != (rows ? WR : p.mode == MODE_LAST ? WL : WC)) return cudaErrorInvalidValue;
     if (p.mode == MODE_LAST) {
-        if (s3_prefetch(p, a)) return launch_s3<L1, L2, L3, WL, false, MODE_LAST, SRC_BUF, true>(p, a, st);
+        if (s3_prefetch(p, a)) return launch_s3<L1, L2, L3, W, false, MODE_LAST, SRC_BUF, true>(p, a, st);
         return dispatch_src<MODE_LAST>(a.src_kind, [&](auto S) {
-            return launch_s3<L1, L2, L3, WL, false, MODE_LAST, decltype(S)::value, false>(p, a, st);
+            return launch_s3<L1, L2, L3, W, false, MODE_LAST, decltype(S)::value, false>(p, a, st);
         });
     }
     return dispatch_mode(p.mode, [&](auto Mc) {
@@ -386,8 +319,8 @@ cudaError_t launch_s3_len(const Pass& p, const PassArgs& a, cudaStream_t st) {
             return cudaErrorInvalidValue;
         } else {
             return dispatch_src<MO>(a.src_kind, [&](auto S) {
-                return rows ? launch_s3<L1, L2, L3, WR, true, MO, decltype(S)::value, false>(p, a, st)
-                            : launch_s3<L1, L2, L3, WC, false, MO, decltype(S)::value, false>(p, a, st);
+                return rows ? launch_s3<L1, L2, L3, W, true, MO, decltype(S)::value, false>(p, a, st)
+                            : launch_s3<L1, L2, L3, W, false, MO, decltype(S)::value, false>(p, a, st);
             });
         }
     });
@@ -395,16 +328,16 @@ cudaError_t launch_s3_len(const Pass& p, const PassArgs& a, cudaStream_t st) {
 
 // occupancy of the form a LAST pass reading src_kind launches (the prefetch form
 // for the scratch buffer)
-template <int L1, int L2, int L3, int WL>
+template <int L1, int L2, int L3, int W>
 cudaError_t s3_last_occupancy_len(const Pass& p, int src_kind, int* blocks_per_sm) {
     return dispatch_src<MODE_LAST>(src_kind, [&](auto S) {
         constexpr int SK = decltype(S)::value;
         constexpr bool PF = SK == SRC_BUF;
-        constexpr size_t smem = s3_smem<L1, L2, L3, WL, MODE_LAST, PF>();
-        auto k = pass_smem3<L1, L2, L3, WL, false, MODE_LAST, SK, PF>;
+        constexpr size_t smem = s3_smem<L1, L2, L3, W, PF>();
+        auto k = pass_smem3<L1, L2, L3, W, false, MODE_LAST, SK, PF>;
         cudaError_t e = smem_limit_once((const void*)k, smem);
         if (e != cudaSuccess) return e;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, s3_threads<MODE_LAST>(), smem);
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, kS3Threads, smem);
     });
 }
 
@@ -415,16 +348,12 @@ cudaError_t upload_twiddles_smem3() { return upload_twiddles(); }
 
 bool smem3_supports(int L) { return L == 2048 || L == 4096; }
 
-int smem3_lines(int L, int mode, int64_t inner) {
-    const bool rows = mode != MODE_LAST && inner == 1;
-    if (L == 2048) return rows ? 4 : mode == MODE_LAST ? 4 : 8;
-    return rows ? 2 : mode == MODE_LAST ? 2 : 4;
-}
+int smem3_lines(int L) { return L == 2048 ? 4 : 2; }
 
 cudaError_t launch_smem3(const Pass& p, const PassArgs& a, cudaStream_t st) {
     switch (p.L) {
-        case 2048: return launch_s3_len<16, 16, 8, 8, 4, 4>(p, a, st);
-        case 4096: return launch_s3_len<16, 16, 16, 4, 2, 2>(p, a, st);
+        case 2048: return launch_s3_len<16, 16, 8, 4>(p, a, st);
+        case 4096: return launch_s3_len<16, 16, 16, 2>(p, a, st);
         default: return cudaErrorInvalidValue;
     }
 }
