@@ -140,6 +140,7 @@ __global__ void __launch_bounds__(128) pass_reg_rows(Pass p, PassArgs a) {
         for (int q = 0; q < Q; ++q) row[q] = v[brev(FWD ? q : (q - (L / 2 - 1) + L) % L, LOG)];
     }
     __syncthreads();
+#pragma unroll 8
     for (int e = tid; e < count * Q; e += LINES) {
         const int l = e / Q, q = e - l * Q;
         const float2 x = rows_sm[l * PITCH + q];
