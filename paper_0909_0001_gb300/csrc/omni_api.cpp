@@ -993,6 +993,8 @@ omni_status run_inverse(omni_plan* pl, double2* V, cudaStream_t st) {
                 a.V = V;
                 a.V_stride = pl->g.Q;
                 a.scale = pl->inv_scale;
+                int e = 0;
+                if (std::frexp(pl->inv_scale, &e) == 0.5) a.scale_shift = 1 - e;  // 2^(e - 1)
             } else {
                 a.dst = dst;
                 a.dst_stride = p.outer * p.q_out * p.inner;

@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(256) pass_direct(Pass p, PassArgs a) {
         }
         const int64_t e = (o * (int64_t)Q + q) * inner + i;
         if constexpr (MODE == MODE_INV_LAST) {
-            a.V[(a.c0 + s) * a.V_stride + e] = make_double2((double)sum.x * a.scale, -(double)sum.y * a.scale);
+            a.V[(a.c0 + s) * a.V_stride + e] = visibility(sum, a);
         } else {
             a.dst[s * a.dst_stride + e] = sum;
         }
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(256, 3) pass_dft(Pass p, PassArgs a) {
                         } else if (db[line] >= 0) {
                             const int64_t at = db[line] + (int64_t)q * inner;
                             if constexpr (MODE == MODE_INV_LAST)
-                                a.V[at] = make_double2((double)v.x * a.scale, -(double)v.y * a.scale);
+                                a.V[at] = visibility(v, a);
                             else
                                 a.dst[at] = v;
                         }
@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(256, 3) pass_dft(Pass p, PassArgs a) {
             if (db[l] < 0) continue;
             const float2 v = ob[l * op + q];
             if constexpr (MODE == MODE_INV_LAST)
-                a.V[db[l] + q] = make_double2((double)v.x * a.scale, -(double)v.y * a.scale);
+                a.V[db[l] + q] = visibility(v, a);
             else if constexpr (MODE != MODE_LAST)
                 a.dst[db[l] + q] = v;
         }

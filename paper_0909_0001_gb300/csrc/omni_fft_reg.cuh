@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(256) pass_reg(Pass p, PassArgs a) {
 #pragma unroll
                 for (int q = 0; q < Q; ++q) {
                     const float2 x = v[brev((q - SH + L) % L, LOG)];
-                    d[(int64_t)q * inner] = make_double2((double)x.x * a.scale, -(double)x.y * a.scale);
+                    d[(int64_t)q * inner] = visibility(x, a);
                 }
             }
         }
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(128) pass_reg_rows(Pass p, PassArgs a) {
         const int l = e / Q, q = e - l * Q;
         const float2 x = rows_sm[l * PITCH + q];
         if constexpr (MODE == MODE_INV_LAST)
-            a.V[to[l] + q] = make_double2((double)x.x * a.scale, -(double)x.y * a.scale);
+            a.V[to[l] + q] = visibility(x, a);
         else
             a.dst[to[l] + q] = x;
     }

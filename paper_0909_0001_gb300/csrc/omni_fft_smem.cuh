@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(256) pass_smem(Pass p, PassArgs a) {
                             a.dst[s * a.dst_stride + (oo * (int64_t)Q + q) * inner + ii] = x;
                         } else {
                             a.V[(a.c0 + s) * a.V_stride + (oo * (int64_t)Q + q) * inner + ii] =
-                                make_double2((double)x.x * a.scale, -(double)x.y * a.scale);
+                                visibility(x, a);
                         }
                     }
                 }

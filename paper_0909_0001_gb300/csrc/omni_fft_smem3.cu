@@ -248,8 +248,8 @@ __global__ void __launch_bounds__(kS3Threads, 2) pass_smem3(Pass p, PassArgs a) 
                     const int64_t second = at + (ROWS ? Q : 1);
                     if constexpr (MODE == MODE_INV_LAST) {
                         double2* V = a.V + (a.c0 + s) * a.V_stride;
-                        if (ok0) V[at] = make_double2((double)re.x * a.scale, -(double)im.x * a.scale);
-                        if (ok1) V[second] = make_double2((double)re.y * a.scale, -(double)im.y * a.scale);
+                        if (ok0) V[at] = visibility(make_float2(re.x, im.x), a);
+                        if (ok1) V[second] = visibility(make_float2(re.y, im.y), a);
                     } else {
                         float2* d = a.dst + s * a.dst_stride;
                         if (ok0) d[at] = make_float2(re.x, im.x);

@@ -84,6 +84,7 @@ struct PassArgs {
     double2* V;          // INV_LAST output
     int64_t V_stride;    // lags per channel
     double scale;        // INV_LAST: 1/L
+    int scale_shift;     // ... k > 0 where it is 2^-k (0: any value)
     int* err;            // device error word (bounded waits that expired set it to 1)
     int force_expire;    // test hook: make the first bounded wait expire
     double fold_scale;   // FP32 LAST passes: factor on the FP64 fold (0 means 1)
