@@ -664,13 +664,14 @@ void choose_chunks(omni_plan* pl) {
         pl->Tc = std::max<int64_t>(1, std::min<int64_t>(1024, cap / per_sample));
         const int64_t cmax = std::min<int64_t>(pl->C, std::max<int64_t>(1, cap / (per_sample * pl->Tc)));
         const int64_t sl = sms > 0 ? (int64_t)sms * std::max(per_sm, 1) : 152;
-        // a chunk's launches, gaps and ramps cost about a quarter of a wave (50 tiles of 12 x 12
-        // antennas, 16 channels x 500 samples: 16 one-channel chunks 4.3 ms, one chunk 3.6)
+        // the launches, gaps and ramps of a chunk of few waves cost about a quarter of a wave; of
+        // more, smaller chunks let host copies overlap (50 tiles of 12 x 12
+        // antennas, 16 channels x 500 samples: 16 one-channel chunks 4.3 ms, one 3.6)
         int64_t best = 1, best_cost = INT64_MAX;
         for (int64_t cc = 1; cc <= cmax; ++cc) {
             const int64_t n = (pl->C + cc - 1) / cc, cb = (pl->C + n - 1) / n, tail = pl->C - (n - 1) * cb;
             const int64_t waves = (n - 1) * ((cb * ctas + sl - 1) / sl) + (tail * ctas + sl - 1) / sl;
-            const int64_t cost = 4 * waves + n;
+            const int64_t cost = 4 * waves + (cb * ctas < 4 * sl ? n : 0);
             if (cost < best_cost) best = cc, best_cost = cost;
         }
         pl->Cc = best;

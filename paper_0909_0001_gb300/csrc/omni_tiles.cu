@@ -49,14 +49,15 @@ struct XSplit {
     bool tri;
 };
 __host__ __device__ inline int xs_first_col(int rb) { return rb * kXA / kXB; }
-__host__ __device__ inline XSplit xsplit(int NT) {
+// warps: of a triangular split's CTAs, 0 for as many as fit.
+__host__ __device__ inline XSplit xsplit(int NT, int warps = 0) {
     XSplit x{};
     x.G = (NT + kXG - 1) / kXG;
     x.tri = NT <= kXRows;
     if (x.tri) {
         const int pairs = x.G * (x.G + 1) / 2;
-        x.parts = (pairs + kXWarps - 1) / kXWarps;
-        x.warps = (pairs + x.parts - 1) / x.parts;
+        x.parts = (pairs + (warps ? warps : kXWarps) - 1) / (warps ? warps : kXWarps);
+        x.warps = warps ? warps : (pairs + x.parts - 1) / x.parts;
     } else {
         const int rows = (x.G + kXA - 1) / kXA, cols = (x.G + kXB - 1) / kXB;
         for (int rb = 0; rb < rows; ++rb) x.parts += cols - xs_first_col(rb);
@@ -89,7 +90,7 @@ __global__ void __launch_bounds__(kXWarps * 32, 1) xspec(Pass p, PassArgs a, con
     const int NT = (int)p.outer;
     const int64_t K = p.L;
     const int64_t ktiles = (K + kXK - 1) / kXK;
-    const XSplit xs = xsplit(NT);
+    const XSplit xs = xsplit(NT, NT <= kXRows ? blockDim.x / 32 : 0);
     int64_t b = blockIdx.x;
     const int part = (int)(b % xs.parts);
     b /= xs.parts;
@@ -261,10 +262,14 @@ cudaError_t xspec_occupancy(const Pass& p, int* blocks_per_sm) {
 
 cudaError_t launch_xspec(const Pass& p, const PassArgs& a, cudaStream_t st) {
     if (a.src_kind != SRC_BUF || !a.err) return cudaErrorInvalidValue;
-    const int64_t blocks = a.S * xspec_ctas_per_channel(p);
-    if (blocks <= 0 || a.tc <= 0) return cudaSuccess;
+    const int64_t ktiles = (p.L + kXK - 1) / kXK;
+    if (a.S <= 0 || a.tc <= 0) return cudaSuccess;
     const int NT = (int)p.outer;
-    const XSplit xs = xsplit(NT);
+    XSplit xs = xsplit(NT);
+    // fewer CTAs than SMs: fewer warps each (one channel of 25 tiles of 8 x 8, 166 samples: 8
+    // CTAs of 10 warps 191 us a pass, the 2 x 16 form 155, this 145)
+    while (xs.tri && xs.warps > 1 && a.S * ktiles * xs.parts < 152) xs = xsplit(NT, (xs.warps + 1) / 2);
+    const int64_t blocks = a.S * ktiles * xs.parts;
     const size_t smem = xs_smem(NT);
     // tensor maps want 16-byte aligned rows; an odd K is a tile of one antenna
     const bool tma = p.L % 2 == 0 && reinterpret_cast<uintptr_t>(a.src) % 16 == 0;
