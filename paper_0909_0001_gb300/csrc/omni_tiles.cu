@@ -203,6 +203,9 @@ __global__ void __launch_bounds__(kXWarps * 32, 1) xspec(Pass p, PassArgs a, con
                 }
             }
         }
+        // these loads come before the box that takes the buffer after the next barrier (the
+        // asynchronous proxy's writes are not ordered behind them by the barrier alone)
+        if constexpr (TMA) fence_async_smem();
     }
     if constexpr (TMA) {
         // no box is in flight when the CTA leaves (each was waited for above unless a wait gave up)

@@ -33,6 +33,9 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, long lo
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(smem_u32(bar)), "r"(bytes));
 }
+// Orders this thread's shared-memory accesses so far before asynchronous copies that a
+// later barrier lets another thread issue (a stage that is read, then filled again).
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 // One box of the 3-D tensor map into shared memory, completing on bar.
 __device__ __forceinline__ void tma_load3(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
     asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
