@@ -39,34 +39,63 @@ constexpr size_t kXBar = 128;    // the stages' barriers, before the stages
 static_assert((kXA + kXB) * kXG <= kXRows && kXA * kXB == kXWarps, "rectangular split");
 static_assert(kXBar + (size_t)kXStages * kXSamples * kXRows * kXK * 8 <= 227 * 1024, "shared memory of one CTA");
 
-// How the pairs of groups gi <= gj are split over CTAs and warps.  Up to 64 tiles a
-// CTA reads every tile and its warps take consecutive pairs of the triangle; beyond,
-// a CTA takes kXA x kXB groups (24 + 32 tiles) touching the triangle.
+// How the pairs of groups gi <= gj are split over CTAs and warps.  XS_FULL: up to 64
+// tiles a CTA reads every tile and its warps take consecutive pairs of the triangle;
+// beyond, a CTA takes kXA x kXB groups (24 + 32 tiles) touching the triangle.  XS_QUAD,
+// XS_PAIR: rectangles of 2 x 2 groups and single pairs of groups, for grids that would
+// leave SMs idle.
+enum XForm : int { XS_FULL = 0, XS_QUAD = 1, XS_PAIR = 2 };
 struct XSplit {
     int G;      // groups
     int parts;  // CTAs per (channel, frequency tile)
     int warps;  // per CTA
+    int A, B;   // rectangle: groups i x groups j
     bool tri;
+    __host__ __device__ int first_col(int rb) const { return rb * A / B; }
+    // stage rows per sample: tiles i and, apart from them, tiles j (0: the same rows)
+    __host__ __device__ int rows_i(int NT) const { return tri ? NT : A * kXG; }
+    __host__ __device__ int rows_j() const { return tri ? 0 : B * kXG; }
+    __host__ __device__ int rows() const { return tri ? G * kXG : (A + B) * kXG; }
+    size_t smem() const { return kXBar + (size_t)kXStages * kXSamples * rows() * kXK * sizeof(float2); }
 };
-__host__ __device__ inline int xs_first_col(int rb) { return rb * kXA / kXB; }
-// warps: of a triangular split's CTAs, 0 for as many as fit.
-__host__ __device__ inline XSplit xsplit(int NT, int warps = 0) {
+__host__ __device__ inline XSplit xsplit(int NT, int form) {
     XSplit x{};
     x.G = (NT + kXG - 1) / kXG;
-    x.tri = NT <= kXRows;
+    x.tri = form == XS_FULL && NT <= kXRows;
     if (x.tri) {
         const int pairs = x.G * (x.G + 1) / 2;
-        x.parts = (pairs + (warps ? warps : kXWarps) - 1) / (warps ? warps : kXWarps);
-        x.warps = warps ? warps : (pairs + x.parts - 1) / x.parts;
+        x.parts = (pairs + kXWarps - 1) / kXWarps;
+        x.warps = (pairs + x.parts - 1) / x.parts;
     } else {
-        const int rows = (x.G + kXA - 1) / kXA, cols = (x.G + kXB - 1) / kXB;
-        for (int rb = 0; rb < rows; ++rb) x.parts += cols - xs_first_col(rb);
-        x.warps = kXWarps;
+        x.A = form == XS_FULL ? kXA : form == XS_QUAD ? 2 : 1;
+        x.B = form == XS_FULL ? kXB : x.A;
+        const int rows = (x.G + x.A - 1) / x.A, cols = (x.G + x.B - 1) / x.B;
+        for (int rb = 0; rb < rows; ++rb) x.parts += cols - x.first_col(rb);
+        x.warps = x.A * x.B;
     }
     return x;
 }
-inline int xs_rows(int NT) { return NT <= kXRows ? (NT + kXG - 1) / kXG * kXG : (kXA + kXB) * kXG; }
-inline size_t xs_smem(int NT) { return kXBar + (size_t)kXStages * kXSamples * xs_rows(NT) * kXK * sizeof(float2); }
+
+// XS_FULL where it gives every SM a CTA; else the form whose busiest SM has the least to
+// do: the warps that each of its four schedulers runs, but no less than the 1.5 times as
+// long that a warp alone takes, for each set of CTAs that fits (ties: the form that loads
+// less).  With XS_FULL alone, its CTAs cut to fewer warps that each still read every tile:
+// 64 tiles of 8 x 8, one channel of 64 samples, 172 -> 125 us a pass; 64 of 4 x 4, 4
+// channels of 512, 441 -> 266; 90 of 2 x 2, 4 channels of 512, 410 -> 237 (a 2 x 16 block
+// of pairs per thread: 127, 319 and 283).
+inline int xs_form(int NT, int64_t units) {
+    const int64_t sms = 152;
+    int best = XS_FULL;
+    if (units * xsplit(NT, XS_FULL).parts >= sms) return best;
+    double least = 0.0;
+    for (int form = XS_FULL; form <= XS_PAIR; ++form) {
+        const XSplit x = xsplit(NT, form);
+        const int64_t each = (units * x.parts + sms - 1) / sms, resident = (int64_t)(227 * 1024 / x.smem());
+        const double t = std::max((double)((each * x.warps + 3) / 4), 1.5 * (double)((each + resident - 1) / resident));
+        if (form == XS_FULL || t < least) best = form, least = t;
+    }
+    return best;
+}
 
 // float -> double where the sums are folded: as plain conversions the compiler moved
 // all 128 of them above the bounds checks and spilled 700 bytes
@@ -79,9 +108,12 @@ __device__ __forceinline__ double widen(float x) {
 // CTA = (channel of the chunk, frequency tile, part of the pairs); the parts of one
 // frequency tile are adjacent, so that they read its spectra from L2.  TMA: one
 // thread brings each stage in with tensor-map boxes two stages ahead (K even: 16-byte
-// rows); else every thread loads the stage (a tile of one antenna, K = 1).
+// rows); else every thread loads the stage (a tile of one antenna, K = 1).  What a stage
+// has no value for (tiles past the last, lanes past K) is whatever shared memory held:
+// those sums are not written.
 template <bool TMA>
-__global__ void __launch_bounds__(kXWarps * 32, 1) xspec(Pass p, PassArgs a, const __grid_constant__ CUtensorMap map0,
+__global__ void __launch_bounds__(kXWarps * 32, 1) xspec(Pass p, PassArgs a, int form,
+                                                         const __grid_constant__ CUtensorMap map0,
                                                          const __grid_constant__ CUtensorMap map1) {
     extern __shared__ __align__(128) unsigned char dsm[];
     uint64_t* full = reinterpret_cast<uint64_t*>(dsm);  // [kXStages], then one that nothing arrives on (test hook)
@@ -90,16 +122,15 @@ __global__ void __launch_bounds__(kXWarps * 32, 1) xspec(Pass p, PassArgs a, con
     const int NT = (int)p.outer;
     const int64_t K = p.L;
     const int64_t ktiles = (K + kXK - 1) / kXK;
-    const XSplit xs = xsplit(NT, NT <= kXRows ? blockDim.x / 32 : 0);
+    const XSplit xs = xsplit(NT, form);
     int64_t b = blockIdx.x;
     const int part = (int)(b % xs.parts);
     b /= xs.parts;
     const int64_t kt = b % ktiles, cc = b / ktiles;
-    // this warp's groups, and the stage rows that hold their tiles: rows 0 .. n0 - 1 are
-    // tiles t0 .., rows n0 .. are tiles t1 ..
+    // this warp's groups, and the stage rows that hold their tiles: n0 rows of tiles t0 .. for
+    // each of the stage's samples, then n1 rows of tiles t1 .. for each
     int gi, gj, ri, rj, t0 = 0, t1 = 0;
-    const int n0 = xs.tri ? NT : kXA * kXG, n1 = xs.tri ? 0 : kXB * kXG;
-    const int rows = xs.tri ? xs.G * kXG : n0 + n1;  // per sample; TMA boxes are n0 + n1 rows, packed
+    const int n0 = xs.rows_i(NT), n1 = xs.rows_j();
     bool live;
     if (xs.tri) {
         int q = part * xs.warps + warp;
@@ -111,20 +142,21 @@ __global__ void __launch_bounds__(kXWarps * 32, 1) xspec(Pass p, PassArgs a, con
         ri = gi * kXG;
         rj = gj * kXG;
     } else {
-        const int cols = (xs.G + kXB - 1) / kXB;
+        const int cols = (xs.G + xs.B - 1) / xs.B;
         int rb = 0, q = part;
-        while (q >= cols - xs_first_col(rb)) q -= cols - xs_first_col(rb++);
-        const int cb = xs_first_col(rb) + q;
-        t0 = rb * kXA * kXG;
-        t1 = cb * kXB * kXG;
-        ri = (warp / kXB) * kXG;
-        rj = n0 + (warp % kXB) * kXG;
-        gi = rb * kXA + warp / kXB;
-        gj = cb * kXB + warp % kXB;
+        while (q >= cols - xs.first_col(rb)) q -= cols - xs.first_col(rb++);
+        const int cb = xs.first_col(rb) + q;
+        t0 = rb * xs.A * kXG;
+        t1 = cb * xs.B * kXG;
+        ri = (warp / xs.B) * kXG;
+        rj = (warp % xs.B) * kXG;
+        gi = rb * xs.A + warp / xs.B;
+        gj = cb * xs.B + warp % xs.B;
         live = gi <= gj && gj < xs.G;
     }
-    const int prow = TMA ? n0 + n1 : rows;  // stage rows per sample
-    const int64_t stage_elems = (int64_t)kXSamples * rows * kXK;
+    const int jn = n1 ? n1 : n0;  // rows of tiles j per sample, and where they begin
+    const int jofs = n1 ? kXSamples * n0 * kXK : 0;
+    const int64_t stage_elems = (int64_t)kXSamples * xs.rows() * kXK;
     const int tc = a.tc, stages = (tc + kXSamples - 1) / kXSamples;
     const long long budget = a.force_expire ? kTestWaitCycles : kWaitCycles;
     if (tid == 0) {
@@ -139,24 +171,19 @@ __global__ void __launch_bounds__(kXWarps * 32, 1) xspec(Pass p, PassArgs a, con
                 uint64_t* bar = full + n % kXStages;
                 mbar_expect_tx(bar, (uint32_t)((n0 + n1) * kXK * kXSamples * sizeof(float2)));
                 const int x = (int)(2 * kXK * kt), z = (int)(cc * tc + n * kXSamples);
-                if (n1 == 0) {
-                    tma_load3(dst, &map0, x, 0, z, bar);
-                } else {  // one box per sample and tile range: the two ranges of a sample are adjacent
-                    for (int s = 0; s < kXSamples; ++s) {
-                        tma_load3(dst + (int64_t)s * prow * kXK, &map0, x, t0, z + s, bar);
-                        tma_load3(dst + ((int64_t)s * prow + n0) * kXK, &map1, x, t1, z + s, bar);
-                    }
-                }
+                tma_load3(dst, &map0, x, t0, z, bar);
+                if (n1) tma_load3(dst + jofs, &map1, x, t1, z, bar);
             }
         } else {
-            for (int e = tid; e < stage_elems; e += blockDim.x) {
-                const int k = e % kXK, r = (e / kXK) % rows, s = e / (kXK * rows);
+            const int nk = (int)(K - kt * kXK < kXK ? K - kt * kXK : kXK), nr = n0 + n1;
+            const int ns = min(kXSamples, tc - n * kXSamples);
+            for (int e = tid; e < nk * nr * ns; e += blockDim.x) {
+                const int k = e % nk, r = (e / nk) % nr, s = e / (nk * nr);
                 const int tile = r < n0 ? t0 + r : t1 + r - n0;
-                const int ts = n * kXSamples + s;
-                const bool in = kt * kXK + k < K && tile < NT && ts < tc;
-                dst[e] = in ? __ldg(reinterpret_cast<const float2*>(a.src) + src_base(a, cc * tc + ts) + tile * K +
-                                    kt * kXK + k)
-                            : make_float2(0.f, 0.f);
+                float2* d = dst + (r < n0 ? (s * n0 + r) * kXK : jofs + (s * n1 + r - n0) * kXK) + k;
+                if (tile < NT)
+                    *d = __ldg(reinterpret_cast<const float2*>(a.src) + src_base(a, cc * tc + n * kXSamples + s) +
+                               (int64_t)tile * K + kt * kXK + k);
             }
         }
     };
@@ -187,8 +214,8 @@ __global__ void __launch_bounds__(kXWarps * 32, 1) xspec(Pass p, PassArgs a, con
         if (live && !failed) {
 #pragma unroll 1
             for (int s = 0; s < ns; ++s) {
-                const float2* yr = st + (s * prow + ri) * kXK;
-                const float2* zr = st + (s * prow + rj) * kXK;
+                const float2* yr = st + (s * n0 + ri) * kXK;
+                const float2* zr = st + jofs + (s * jn + rj) * kXK;
                 float2 y[kXG];
 #pragma unroll
                 for (int u = 0; u < kXG; ++u) y[u] = yr[u * kXK];
@@ -253,41 +280,37 @@ __global__ void __launch_bounds__(kXWarps * 32, 1) xspec(Pass p, PassArgs a, con
 }  // namespace
 
 int64_t xspec_ctas_per_channel(const Pass& p) {
-    return ((p.L + kXK - 1) / kXK) * (int64_t)xsplit((int)p.outer).parts;
+    return ((p.L + kXK - 1) / kXK) * (int64_t)xsplit((int)p.outer, XS_FULL).parts;
 }
 
 cudaError_t xspec_occupancy(const Pass& p, int* blocks_per_sm) {
-    const int NT = (int)p.outer;
-    cudaError_t e = smem_limit_once((const void*)xspec<true>, xs_smem(NT));
+    const XSplit xs = xsplit((int)p.outer, XS_FULL);
+    cudaError_t e = smem_limit_once((const void*)xspec<true>, xs.smem());
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, xspec<true>, 32 * xsplit(NT).warps, xs_smem(NT));
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, xspec<true>, 32 * xs.warps, xs.smem());
 }
 
 cudaError_t launch_xspec(const Pass& p, const PassArgs& a, cudaStream_t st) {
     if (a.src_kind != SRC_BUF || !a.err) return cudaErrorInvalidValue;
     const int64_t ktiles = (p.L + kXK - 1) / kXK;
     if (a.S <= 0 || a.tc <= 0) return cudaSuccess;
-    const int NT = (int)p.outer;
-    XSplit xs = xsplit(NT);
-    // fewer CTAs than SMs: fewer warps each (one channel of 25 tiles of 8 x 8, 166 samples: 8
-    // CTAs of 10 warps 191 us a pass, the 2 x 16 form 155, this 145)
-    while (xs.tri && xs.warps > 1 && a.S * ktiles * xs.parts < 152) xs = xsplit(NT, (xs.warps + 1) / 2);
+    const int NT = (int)p.outer, form = xs_form(NT, a.S * ktiles);
+    const XSplit xs = xsplit(NT, form);
     const int64_t blocks = a.S * ktiles * xs.parts;
-    const size_t smem = xs_smem(NT);
     // tensor maps want 16-byte aligned rows; an odd K is a tile of one antenna
     const bool tma = p.L % 2 == 0 && reinterpret_cast<uintptr_t>(a.src) % 16 == 0;
     CUtensorMap m0{}, m1{};
     if (tma) {
         const int64_t samples = a.S * a.tc;
-        cudaError_t e = xs.tri ? encode_spectra_map(a.src, p.L, NT, samples, 2 * kXK, NT, kXSamples, &m0)
-                               : encode_spectra_map(a.src, p.L, NT, samples, 2 * kXK, kXA * kXG, 1, &m0);
-        if (e == cudaSuccess && !xs.tri) e = encode_spectra_map(a.src, p.L, NT, samples, 2 * kXK, kXB * kXG, 1, &m1);
+        cudaError_t e = encode_spectra_map(a.src, p.L, NT, samples, 2 * kXK, xs.rows_i(NT), kXSamples, &m0);
+        if (e == cudaSuccess && !xs.tri)
+            e = encode_spectra_map(a.src, p.L, NT, samples, 2 * kXK, xs.rows_j(), kXSamples, &m1);
         if (e != cudaSuccess) return e;
     }
     auto kern = tma ? xspec<true> : xspec<false>;
-    cudaError_t e = smem_limit_once((const void*)kern, smem);
+    cudaError_t e = smem_limit_once((const void*)kern, xs.smem());
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)blocks, 32 * xs.warps, smem, st>>>(p, a, m0, m1);
+    kern<<<(unsigned)blocks, 32 * xs.warps, xs.smem(), st>>>(p, a, form, m0, m1);
     return cudaGetLastError();
 }
 
