@@ -378,7 +378,7 @@ void use_smem3(Pass& p, const Knobs& k) {
     const bool fwd = p.mode == MODE_MID || p.mode == MODE_LAST;
     if (fwd && 2 * p.n > p.L) return;
     p.kind = KIND_SMEM3;
-    p.W = smem3_lines(p.L);
+    p.W = smem3_lines(p);
 }
 
 // FP64 values of one channel's accumulator: |F|^2 over the padded lattice, or

@@ -11,7 +11,8 @@
 // (the factorisation of w_L^(j k) into the three DFTs and two twiddle stages).
 // The inverse passes use the same transform (the inverse runs as a forward FFT)
 // on all L inputs and keep the lag slots, the last one conjugated and scaled.
-// A 256-thread CTA, two per SM, transforms W lines in pairs: each shared-memory element
+// A 256-thread CTA, two per SM (one of 512 where four lines of 4096 points go together),
+// transforms W lines in pairs: each shared-memory element
 // is one point of two lines (re, re, im, im), so that a point is one 16-byte access, the
 // butterflies run on both lines per f32x2 instruction and the twiddle powers are formed
 // once for both.  A line pair is held as [j1][j2][j3] with a row pitch L3 + 1, so that
@@ -34,7 +35,11 @@
 namespace omni {
 namespace {
 
-constexpr int kS3Threads = 256;
+// lines per CTA (see smem3_lines)
+constexpr int kS3W2048 = 4, kS3W4096 = 2, kS3W4096Strided = 4;
+
+// one step-1 task (16 points of a line pair) per thread
+constexpr int s3_threads(int L, int W) { return W / 2 * L / 16; }
 
 template <int L1, int L2, int L3>
 struct S3Geom {
@@ -92,14 +97,15 @@ __device__ __forceinline__ void cmul2(f2x& x, f2x& y, float2 w) {
 // sample's W x L/2 inputs are copied asynchronously into a staging buffer
 // [j][W] while the current sample runs steps 2 and 3, and step 1 reads them there.
 template <int L1, int L2, int L3, int W, bool ROWS, int MODE, int SRC, bool PF>
-__global__ void __launch_bounds__(kS3Threads, 2) pass_smem3(Pass p, PassArgs a) {
+__global__ void __launch_bounds__(s3_threads(L1 * L2 * L3, W), 512 / s3_threads(L1 * L2 * L3, W)) pass_smem3(Pass p, PassArgs a) {
     using G = S3Geom<L1, L2, L3>;
     static_assert(!PF || (MODE == MODE_LAST && SRC == SRC_BUF && !ROWS), "prefetch form");
     constexpr int L = G::L, M = G::M, P1 = G::P1, P2 = G::P2, PLANE = G::PLANE;
     constexpr bool FWD = MODE == MODE_MID || MODE == MODE_LAST;  // forward: inputs j >= L/2 are zero
     constexpr int LOG1 = ilog2(L1), LOG2 = ilog2(L2), LOG3 = ilog2(L3), H = W / 2;
-    static_assert(W % 2 == 0 && H * M == kS3Threads && H * L1 * L3 == kS3Threads, "one task per thread, steps 1 and 2");
-    constexpr int T3 = H * L1 * L2 / kS3Threads;  // step-3 tasks per thread
+    constexpr int NT = s3_threads(L, W);
+    static_assert(W % 2 == 0 && H * M == NT && H * L1 * L3 == NT, "one task per thread, steps 1 and 2");
+    constexpr int T3 = H * L1 * L2 / NT;  // step-3 tasks per thread
     extern __shared__ float4 sm4[];
     float4* lines = sm4;                                            // [H][PLANE]
     float2* stage = reinterpret_cast<float2*>(lines + H * PLANE);   // PF: [L/2][W]
@@ -141,11 +147,11 @@ __global__ void __launch_bounds__(kS3Threads, 2) pass_smem3(Pass p, PassArgs a) 
     // past the axis are zero-filled
     auto prefetch = [&](int64_t s) {
         const float2* row0 = reinterpret_cast<const float2*>(a.src) + s * a.src_stride + i0;
-        constexpr int NC = (L / 2) * H / kS3Threads;
-        static_assert(NC * kS3Threads == (L / 2) * H, "copies per thread");
+        constexpr int NC = (L / 2) * H / NT;
+        static_assert(NC * NT == (L / 2) * H, "copies per thread");
 #pragma unroll
         for (int r = 0; r < NC; ++r) {
-            const int c = tid + r * kS3Threads, j = c / H, h = c % H;
+            const int c = tid + r * NT, j = c / H, h = c % H;
             const bool ok = j < n && i0 + 2 * h < inner;
             cp_async16(stage + j * W + 2 * h, ok ? row0 + (int64_t)j * inner + 2 * h : row0, ok);
         }
@@ -224,7 +230,7 @@ __global__ void __launch_bounds__(kS3Threads, 2) pass_smem3(Pass p, PassArgs a) 
         // k3 are consecutive bins and go straight out
 #pragma unroll
         for (int u = 0; u < T3; ++u) {
-            const int t = tid + u * kS3Threads;
+            const int t = tid + u * NT;
             const int h = ROWS ? t / (L1 * L2) : t % H, k12 = ROWS ? t % (L1 * L2) : t / H, k1 = k12 % L1, k2 = k12 / L1;
             const float4* r = lines + h * PLANE + k1 * P1 + k2 * P2;
             f2x x[L3], y[L3];
@@ -264,7 +270,7 @@ __global__ void __launch_bounds__(kS3Threads, 2) pass_smem3(Pass p, PassArgs a) 
     if constexpr (MODE == MODE_LAST) {
 #pragma unroll
         for (int u = 0; u < T3; ++u) {
-            const int t = tid + u * kS3Threads, h = t % H, k12 = t / H;
+            const int t = tid + u * NT, h = t % H, k12 = t / H;
 #pragma unroll
             for (int k3 = 0; k3 < L3; ++k3) {
                 const float2 v = unpack2(acc[u][k3]);
@@ -297,15 +303,16 @@ cudaError_t launch_s3(const Pass& p, const PassArgs& a, cudaStream_t st) {
     auto k = pass_smem3<L1, L2, L3, W, ROWS, MODE, SRC, PF>;
     cudaError_t e = smem_limit_once((const void*)k, smem);
     if (e != cudaSuccess) return e;
-    k<<<MODE == MODE_LAST ? last_grid(blocks, a) : dim3((unsigned)blocks), kS3Threads, smem, st>>>(p, a);
+    k<<<MODE == MODE_LAST ? last_grid(blocks, a) : dim3((unsigned)blocks), s3_threads(L1 * L2 * L3, W), smem, st>>>(p, a);
     return cudaGetLastError();
 }
 
-// one length: W lines along a strided axis or along the innermost axis
-template <int L1, int L2, int L3, int W>
+// one length: W lines in a LAST pass and along the innermost axis, WS in the other passes
+// of a strided axis
+template <int L1, int L2, int L3, int W, int WS>
 cudaError_t launch_s3_len(const Pass& p, const PassArgs& a, cudaStream_t st) {
     const bool fwd = p.mode == MODE_MID || p.mode == MODE_LAST;
-    if (p.n > (fwd ? L1 * L2 * L3 / 2 : L1 * L2 * L3) || p.W != W) return cudaErrorInvalidValue;
+    if (p.n > (fwd ? L1 * L2 * L3 / 2 : L1 * L2 * L3) || p.W != smem3_lines(p)) return cudaErrorInvalidValue;
     const bool rows = p.mode != MODE_LAST && p.inner == 1;
     if (p.mode == MODE_LAST) {
         if (s3_prefetch(p, a)) return launch_s3<L1, L2, L3, W, false, MODE_LAST, SRC_BUF, true>(p, a, st);
@@ -320,7 +327,7 @@ cudaError_t launch_s3_len(const Pass& p, const PassArgs& a, cudaStream_t st) {
         } else {
             return dispatch_src<MO>(a.src_kind, [&](auto S) {
                 return rows ? launch_s3<L1, L2, L3, W, true, MO, decltype(S)::value, false>(p, a, st)
-                            : launch_s3<L1, L2, L3, W, false, MO, decltype(S)::value, false>(p, a, st);
+                            : launch_s3<L1, L2, L3, WS, false, MO, decltype(S)::value, false>(p, a, st);
             });
         }
     });
@@ -337,7 +344,7 @@ cudaError_t s3_last_occupancy_len(const Pass& p, int src_kind, int* blocks_per_s
         auto k = pass_smem3<L1, L2, L3, W, false, MODE_LAST, SK, PF>;
         cudaError_t e = smem_limit_once((const void*)k, smem);
         if (e != cudaSuccess) return e;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, kS3Threads, smem);
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, s3_threads(L1 * L2 * L3, W), smem);
     });
 }
 
@@ -348,20 +355,26 @@ cudaError_t upload_twiddles_smem3() { return upload_twiddles(); }
 
 bool smem3_supports(int L) { return L == 2048 || L == 4096; }
 
-int smem3_lines(int L) { return L == 2048 ? 4 : 2; }
+// Passes of a strided axis touch memory in runs of 8 W bytes.  4096 points: one line pair,
+// two CTAs per SM, where a LAST pass sums in registers and its loads run ahead; the other
+// passes write every bin and take two pairs, whole 32-byte sectors (8 x 2048 antennas on
+// 2 x 2, 16 channels x 32 samples: MID 1.21 -> 0.89 ms, inverse MID 100 -> 66 us).
+int smem3_lines(const Pass& p) {
+    return p.L == 2048 ? kS3W2048 : p.mode == MODE_LAST || p.inner == 1 ? kS3W4096 : kS3W4096Strided;
+}
 
 cudaError_t launch_smem3(const Pass& p, const PassArgs& a, cudaStream_t st) {
     switch (p.L) {
-        case 2048: return launch_s3_len<16, 16, 8, 4>(p, a, st);
-        case 4096: return launch_s3_len<16, 16, 16, 2>(p, a, st);
+        case 2048: return launch_s3_len<16, 16, 8, kS3W2048, kS3W2048>(p, a, st);
+        case 4096: return launch_s3_len<16, 16, 16, kS3W4096, kS3W4096Strided>(p, a, st);
         default: return cudaErrorInvalidValue;
     }
 }
 
 cudaError_t smem3_last_occupancy(const Pass& p, int src_kind, int* blocks_per_sm) {
     switch (p.L) {
-        case 2048: return s3_last_occupancy_len<16, 16, 8, 4>(p, src_kind, blocks_per_sm);
-        case 4096: return s3_last_occupancy_len<16, 16, 16, 2>(p, src_kind, blocks_per_sm);
+        case 2048: return s3_last_occupancy_len<16, 16, 8, kS3W2048>(p, src_kind, blocks_per_sm);
+        case 4096: return s3_last_occupancy_len<16, 16, 16, kS3W4096>(p, src_kind, blocks_per_sm);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -138,7 +138,7 @@ int64_t xspec_ctas_per_channel(const Pass& p);
 // Three-step passes of 2048 and 4096 points: lines per CTA (W consecutive inner
 // indices, or for an innermost axis W consecutive outer lines).
 bool smem3_supports(int L);
-int smem3_lines(int L);
+int smem3_lines(const Pass& p);
 cudaError_t launch_smem3(const Pass& p, const PassArgs& a, cudaStream_t stream);
 cudaError_t smem3_last_occupancy(const Pass& p, int src_kind, int* blocks_per_sm);
 bool xspec5_supports(int64_t n_tiles, int64_t K);  // <= 64 tiles, K a multiple of 4
