@@ -271,12 +271,38 @@ __global__ void __launch_bounds__(s3_threads(L1 * L2 * L3, W), 512 / s3_threads(
 #pragma unroll
         for (int u = 0; u < T3; ++u) {
             const int t = tid + u * NT, h = t % H, k12 = t / H;
+            const int64_t e0 = (int64_t)k12 * inner + i0 + 2 * h, step = (int64_t)L1 * L2 * inner;
+            if (inner % 2 == 0) {
+                // both lines of the pair, or neither: 16 bytes at a time, loads together (value by
+                // value, each waited for: 16 x 2048 antennas, 16 channels x 4 samples, the pass
+                // 152 us against 56)
+                if (!line_ok(2 * h)) continue;
+                if (gridDim.y > 1) {  // as fold_last
+                    float2* d = reinterpret_cast<float2*>(a.part + ((int64_t)blockIdx.y * a.S + cc) * a.P_stride + e0);
 #pragma unroll
-            for (int k3 = 0; k3 < L3; ++k3) {
-                const float2 v = unpack2(acc[u][k3]);
-                const int64_t at = (int64_t)(k12 + L1 * L2 * k3) * inner + i0 + 2 * h;
-                if (line_ok(2 * h)) fold_last(a, cc, at, v.x);
-                if (line_ok(2 * h + 1)) fold_last(a, cc, at + 1, v.y);
+                    for (int k3 = 0; k3 < L3; ++k3) d[k3 * step / 2] = unpack2(acc[u][k3]);
+                    continue;
+                }
+                double2* P = reinterpret_cast<double2*>(a.P + (a.c0 + cc) * a.P_stride + e0);
+                constexpr int NB = 8;
+#pragma unroll
+                for (int k0 = 0; k0 < L3; k0 += NB) {
+                    double2 s[NB];
+#pragma unroll
+                    for (int k = 0; k < NB; ++k) s[k] = P[(k0 + k) * step / 2];
+#pragma unroll
+                    for (int k = 0; k < NB; ++k) {
+                        const float2 v = unpack2(acc[u][k0 + k]);
+                        P[(k0 + k) * step / 2] = make_double2(s[k].x + (double)v.x, s[k].y + (double)v.y);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int k3 = 0; k3 < L3; ++k3) {
+                    const float2 v = unpack2(acc[u][k3]);
+                    if (line_ok(2 * h)) fold_last(a, cc, e0 + k3 * step, v.x);
+                    if (line_ok(2 * h + 1)) fold_last(a, cc, e0 + k3 * step + 1, v.y);
+                }
             }
         }
     }
