@@ -122,7 +122,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // value for (tiles past the last, lanes past K) is whatever shared memory held: those sums
 // are not written.
 template <bool TMA>
-__global__ void __launch_bounds__(kXWarps * 32, 1) xspec(Pass p, PassArgs a, int form,
+__global__ void __launch_bounds__(kXWarps * 32, 1) xspec(Pass p, PassArgs a, int form, int few,
                                                          const __grid_constant__ CUtensorMap map0,
                                                          const __grid_constant__ CUtensorMap map1) {
     extern __shared__ __align__(128) unsigned char dsm[];
@@ -257,6 +257,29 @@ __global__ void __launch_bounds__(kXWarps * 32, 1) xspec(Pass p, PassArgs a, int
     if (!live || k >= K) return;
     double2* S = reinterpret_cast<double2*>(a.P + (a.c0 + cc) * a.P_stride) + k;
     const int i0 = gi * kXG, j0 = gj * kXG;
+    if (few) {
+        // fewer CTAs than SMs, whose warps would wait for one load after another (9 tiles of
+        // 12 x 12, one channel x 8 samples: the pass 35 us, so 13): reductions in L2, one per
+        // value of a launch, so that the order of the sums stays that of the launches
+#pragma unroll
+        for (int u = 0; u < kXG; ++u)
+#pragma unroll
+            for (int v = 0; v < kXG; ++v) {
+                const int i = i0 + u, j = j0 + v;
+                if (i < NT && j < NT) {
+                    const double re = widen(ar[u][v]), im = widen(ai[u][v]);
+                    double* f = reinterpret_cast<double*>(S + (i * NT + j) * K);
+                    atomicAdd(f, re);
+                    atomicAdd(f + 1, im);
+                    if (gi != gj) {
+                        double* m = reinterpret_cast<double*>(S + (j * NT + i) * K);
+                        atomicAdd(m, re);
+                        atomicAdd(m + 1, -im);
+                    }
+                }
+            }
+        return;
+    }
     // both orders of each pair; kXF of them at a time, their loads together
     constexpr int kXF = 2;
 #pragma unroll
@@ -319,7 +342,7 @@ cudaError_t launch_xspec(const Pass& p, const PassArgs& a, cudaStream_t st) {
     auto kern = tma ? xspec<true> : xspec<false>;
     cudaError_t e = smem_limit_once((const void*)kern, xs.smem());
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)blocks, 32 * xs.warps, xs.smem(), st>>>(p, a, form, m0, m1);
+    kern<<<(unsigned)blocks, 32 * xs.warps, xs.smem(), st>>>(p, a, form, blocks < 152, m0, m1);
     return cudaGetLastError();
 }
 

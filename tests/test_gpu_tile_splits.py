@@ -29,3 +29,16 @@ def test_splits_match_oracle(n1, n2, nt, C, T):
         V = plan.visibilities().reshape(C, -1).cpu().numpy()
     ref = oracle.tile_correlate(n1, n2, nt, x).reshape(C, -1)
     assert (np.linalg.norm(V - ref, axis=1) / np.linalg.norm(ref, axis=1)).max() <= 1e-5
+
+
+@pytest.mark.parametrize("n1, n2, nt, C", [(4, 4, 64, 26), (3, 5, 9, 1), (2, 4, 57, 8), (2, 2, 64, 16), (1, 1, 65, 3)])
+def test_calls_add_up(n1, n2, nt, C):
+    """Each split folds into the sums of the calls before."""
+    x = synth.random_complex([n1, n2, nt], C, 9, seed=1100 + nt)
+    offs = np.random.default_rng(nt).uniform(-900.0, 900.0, size=(nt, 2))
+    with omni.TilePlan(synth.Level(n1, n2, (1.0, 0.3, 0.0, 1.0)), offs, C) as plan:
+        plan.correlate(x[:, :5].contiguous().cuda())
+        plan.correlate(x[:, 5:].contiguous().cuda())
+        V = plan.visibilities().reshape(C, -1).cpu().numpy()
+    ref = oracle.tile_correlate(n1, n2, nt, x).reshape(C, -1)
+    assert (np.linalg.norm(V - ref, axis=1) / np.linalg.norm(ref, axis=1)).max() <= 1e-5
