@@ -13,11 +13,20 @@ namespace omni {
 // ---------------------------------------------------------------- direct DFT passes
 
 // Any length: one thread per output value, X[k] = sum_j x[j] w_L^(jk mod L).
-template <int MODE, int SRC>
+// SLICED (LAST over slices of the samples): four terms' loads together.  Unsliced, one
+// plain loop from sample 0: what the compiler makes of it is 1.4 times as fast as that (500
+// points, 128 columns, 8 samples: 0.19 against 0.27 ms), and 1.8 times as fast as the same
+// loop between two bounds (0.35; in four slices 0.17, four loads together 0.10).  Both in
+// one kernel cost the plain loop a quarter.
+template <int MODE, int SRC, bool SLICED>
 __global__ void __launch_bounds__(256) pass_direct(Pass p, PassArgs a) {
     const int64_t flat = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t inner = p.inner;
     const int L = p.L, n = p.n, Q = p.q_out;
+    auto term = [&](float2& sum, float2 x, float2 w) {
+        sum.x = fmaf(x.x, w.x, fmaf(-x.y, w.y, sum.x));
+        sum.y = fmaf(x.x, w.y, fmaf(x.y, w.x, sum.y));
+    };
     if constexpr (MODE == MODE_LAST) {
         const int64_t per = (int64_t)L * inner;
         if (flat >= a.S * per) return;
@@ -26,21 +35,48 @@ __global__ void __launch_bounds__(256) pass_direct(Pass p, PassArgs a) {
         const int k = (int)(r / inner);
         const int64_t i = r - (int64_t)k * inner;
         float acc = 0.0f;
-        int tb, te;
-        slice_samples(a, tb, te);
-        for (int tt = tb; tt < te; ++tt) {
-            const int64_t base = src_base(a, cc * a.tc + tt) + i;
-            float2 sum = make_float2(0.f, 0.f);
-            int m = 0;
-            for (int j = 0; j < n; ++j) {
-                const float2 x = ld_src<SRC>(a.src, base + (int64_t)j * inner);
-                const float2 w = __ldg(p.tw + m);
-                sum.x = fmaf(x.x, w.x, fmaf(-x.y, w.y, sum.x));
-                sum.y = fmaf(x.x, w.y, fmaf(x.y, w.x, sum.y));
-                m += k;
-                if (m >= L) m -= L;
+        if constexpr (!SLICED) {
+            for (int tt = 0; tt < a.tc; ++tt) {
+                const int64_t base = src_base(a, cc * a.tc + tt) + i;
+                float2 sum = make_float2(0.f, 0.f);
+                int m = 0;
+                for (int j = 0; j < n; ++j) {
+                    const float2 x = ld_src<SRC>(a.src, base + (int64_t)j * inner);
+                    term(sum, x, __ldg(p.tw + m));
+                    m += k;
+                    if (m >= L) m -= L;
+                }
+                acc += cnorm(sum);
             }
-            acc += cnorm(sum);
+        } else {
+            constexpr int NB = 4;
+            int tb, te;
+            slice_samples(a, tb, te);
+#pragma unroll 1
+            for (int tt = tb; tt < te; ++tt) {
+                const int64_t base = src_base(a, cc * a.tc + tt) + i;
+                float2 sum = make_float2(0.f, 0.f);
+                int m = 0, j = 0;
+                for (; j + NB <= n; j += NB) {
+                    float2 x[NB], w[NB];
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) {
+                        x[u] = ld_src<SRC>(a.src, base + (int64_t)(j + u) * inner);
+                        w[u] = __ldg(p.tw + m);
+                        m += k;
+                        if (m >= L) m -= L;
+                    }
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) term(sum, x[u], w[u]);
+                }
+#pragma unroll 1
+                for (; j < n; ++j) {
+                    term(sum, ld_src<SRC>(a.src, base + (int64_t)j * inner), __ldg(p.tw + m));
+                    m += k;
+                    if (m >= L) m -= L;
+                }
+                acc += cnorm(sum);
+            }
         }
         fold_last(a, cc, (int64_t)k * inner + i, acc);
     } else {
@@ -58,9 +94,7 @@ __global__ void __launch_bounds__(256) pass_direct(Pass p, PassArgs a) {
         int m = 0;
         for (int j = 0; j < n; ++j) {
             const float2 x = ld_src<SRC>(a.src, base + (int64_t)j * inner);
-            const float2 w = __ldg(p.tw + m);
-            sum.x = fmaf(x.x, w.x, fmaf(-x.y, w.y, sum.x));
-            sum.y = fmaf(x.x, w.y, fmaf(x.y, w.x, sum.y));
+            term(sum, x, __ldg(p.tw + m));
             m += k;
             if (m >= L) m -= L;
         }
@@ -381,7 +415,10 @@ cudaError_t launch_direct_t(const Pass& p, const PassArgs& a, cudaStream_t st) {
     }
     const int threads = 256;
     const int64_t blocks = (work + threads - 1) / threads;
-    pass_direct<MODE, SRC><<<MODE == MODE_LAST ? last_grid(blocks, a) : dim3((unsigned)blocks), threads, 0, st>>>(p, a);
+    if (MODE == MODE_LAST && a.split > 1)
+        pass_direct<MODE, SRC, MODE == MODE_LAST><<<last_grid(blocks, a), threads, 0, st>>>(p, a);
+    else
+        pass_direct<MODE, SRC, false><<<(unsigned)blocks, threads, 0, st>>>(p, a);
     return cudaGetLastError();
 }
 
