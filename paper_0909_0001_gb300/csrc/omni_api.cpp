@@ -252,8 +252,12 @@ struct omni_plan {
     omni_precision precision = OMNI_FP32;
     std::vector<Pass> fwd, inv;
     int64_t Cc = 1, Tc = 1;   // forward chunk: channels x samples
-    int slices = 1;           // LAST: slices of a chunk's samples (fewer CTAs than the GPU holds)
-    float* part = nullptr;    // ... their sums, [slices][Cc][L]
+    int slices = 1;           // LAST: most slices of a chunk's samples (fewer CTAs than the GPU holds)
+    int64_t last_ctas = 1;    // ... CTAs of the last pass per channel, how many an SM holds, SMs
+    int last_per_sm = 2, sms = 152;
+    float* part = nullptr;    // ... the slices' sums, [slices][Cc][L]
+    int sliced = 1;           // ... slices of chunks of sliced_tc samples
+    int64_t sliced_tc = 0;
     bool beams = false;       // beam-space plan: level-1 axes unpadded, no lag over them
     int64_t n_tiles = 0;      // tile-hybrid plan: identical tiles at arbitrary offsets
     int64_t lag_pairs = 0;    // mixed 2-level plan with a lag-sum level 2: coarse lags kept per
@@ -606,6 +610,31 @@ omni_status build_passes(omni_plan* pl) {
     return OMNI_OK;
 }
 
+// Channels of a call's chunks (equal, but for the last; host input starts with fewer).
+int64_t chunk_channels(const omni_plan* pl) { return ceil_div(pl->C, ceil_div(pl->C, pl->Cc)); }
+
+// Slices of the last pass's tc samples over cc channels: too few CTAs leave the GPU
+// idle, but each slice's sums are written and read again (FFT passes: 8 bytes per point of
+// the lattice, where a sample reads 2 to 4, two samples' time) and one more kernel adds
+// them (six).  The number of least time in whole waves, if a tenth less than unsliced.
+// With a slice's cost taken as a 50th of the pass whatever its samples: three levels of 8 x 8,
+// 8 x 8 and 2 x 2, 16 channels x 4 samples, 1.01 ms a pass, unsliced 0.68.
+int choose_slices(const omni_plan* pl, int64_t cc, int64_t tc, int64_t most) {
+    const Pass& last = pl->fwd.back();
+    LastShape s{cc * pl->last_ctas, pl->last_per_sm, 2.0, 6.0};
+    if (last.kind == KIND_REG) s.ctas = (cc * last.inner + 255) / 256;
+    if (last.kind == KIND_DIRECT) s = direct_last_shape(last, cc);
+    const int64_t slots = pl->sms * s.per_sm;
+    const double fold = s.fold * s.ctas / slots;
+    double best = 0.9 * (double)(tc * ceil_div(s.ctas, slots));
+    int slices = 1;
+    for (int64_t k = 2; k <= std::min(most, tc) && s.ctas < 2 * slots && fold * k + s.launch < best; ++k) {
+        const double t = (double)(ceil_div(tc, k) * ceil_div(s.ctas * k, slots)) + fold * k + s.launch;
+        if (t < best) best = t, slices = (int)k;
+    }
+    return slices;
+}
+
 // Chunk sizes: the last pass gets one wave of resident CTAs (channels x inner
 // tiles), and each scratch buffer holds about chunk_mb MB of samples (3072, the
 // autotuner's pick on the 2-level workload for both paths; OMNI_CHUNK_MB overrides):
@@ -679,18 +708,15 @@ void choose_chunks(omni_plan* pl) {
     if (pl->knobs.chunk_channels > 0) pl->Cc = std::min<int64_t>(pl->C, pl->knobs.chunk_channels);
     const int64_t samples = std::max<int64_t>(1, target / per_sample);
     if (!whole_waves) pl->Tc = std::max<int64_t>(1, std::min<int64_t>(1024, samples / pl->Cc));
-    // too few CTAs for the GPU: cut the samples into slices, the number that takes the
-    // least time in whole waves (a slice's fold counts as a 50th of the pass), within 256 MB of sums
+    // too few CTAs for the GPU: slices of the samples, within 256 MB of sums
     pl->slices = 1;
     if (last.kind == KIND_LEVEL || last.kind == KIND_REG || last.kind == KIND_SMEM || last.kind == KIND_SMEM3 ||
         last.kind == KIND_DIRECT) {
-        const int64_t c = last.kind == KIND_DIRECT ? pl->Cc * ((last.inner + 63) / 64) : pl->Cc * ctas;
-        const int64_t most = std::min<int64_t>((int64_t)64, ((int64_t)256 << 20) / std::max<int64_t>(1, 4 * pl->Cc * acc_doubles(pl)));
-        double best = 1.0 * ceil_div(c, slots);
-        for (int64_t k = 2; k <= most && c < 2 * slots; ++k) {
-            const double t = (double)ceil_div(c * k, slots) / k + 0.02;
-            if (t < 0.9 * best) best = t, pl->slices = (int)k;
-        }
+        pl->last_ctas = ctas;
+        pl->last_per_sm = std::max(per_sm, 2);
+        pl->sms = sms > 0 ? sms : 152;
+        const int64_t bytes = std::max<int64_t>(1, 4 * pl->Cc * acc_doubles(pl));
+        pl->slices = choose_slices(pl, chunk_channels(pl), pl->Tc, std::min<int64_t>(64, ((int64_t)256 << 20) / bytes));
     }
     const int64_t per_chan = std::max<int64_t>(1, pl->inv_elems) * (int64_t)sizeof(float2);
     pl->Cv = std::min<int64_t>(pl->C, std::max<int64_t>(1, target / per_chan));
@@ -914,7 +940,11 @@ omni_status run_chunk(omni_plan* pl, const void* volts, int64_t vc0, int64_t Tsr
         }
         if (p.mode == MODE_LAST) {
             a.S = cc;
-            a.split = (int)std::min<int64_t>(pl->slices, tc);
+            if (pl->slices > 1 && tc != pl->sliced_tc) {
+                pl->sliced = choose_slices(pl, chunk_channels(pl), tc, pl->slices);
+                pl->sliced_tc = tc;
+            }
+            a.split = pl->slices > 1 ? pl->sliced : 1;
             a.part = pl->part;
         } else {
             a.S = cc * tc;
@@ -1674,7 +1704,7 @@ omni_status omni_correlate(omni_plan* pl, const void* volts_dev, int64_t T, void
         for (int b = 0; b < 2; ++b) OMNI_CUDA(cudaEventRecord(pl->last_done[b], s), "cudaEventRecord");
     }
     // equal-sized chunks (no short tail chunk paying a whole fold and launch)
-    const int64_t Cb = ceil_div(pl->C, ceil_div(pl->C, pl->Cc));
+    const int64_t Cb = chunk_channels(pl);
     const int64_t Tb = ceil_div(T, ceil_div(T, pl->Tc));
     int64_t j = 0;
     for (int64_t c0 = 0; c0 < pl->C; c0 += Cb) {
@@ -1744,7 +1774,7 @@ omni_status omni_correlate_host(omni_plan* pl, const void* volts_host, int64_t T
     // first chunk's copy, and each next copy (host copies ran at 210 GB/s, about
     // three quarters of the transforms' rate on the 2-level workload) must fit in
     // the previous chunk's transforms, so the channel count grows by 30% a chunk
-    const int64_t Cb = ceil_div(pl->C, ceil_div(pl->C, pl->Cc));
+    const int64_t Cb = chunk_channels(pl);
     const int64_t Tb = ceil_div(T, ceil_div(T, pl->Tc));
     int64_t next = std::max<int64_t>(1, Cb / 4);
     int64_t j = 0;

@@ -385,12 +385,21 @@ __global__ void __launch_bounds__(256, 3) pass_dft(Pass p, PassArgs a) {
 
 namespace {
 
+// The tiled form of a pass: padded lines (HALF) or whole lines, up to kDftMax points as
+// shared memory allows; false: none.
+bool dft_form(const Pass& p, DftShape* d, bool* half) {
+    if (p.L < 2 || p.L > kDftMax) return false;
+    const bool fwd = p.mode == MODE_MID || p.mode == MODE_LAST;
+    *half = fwd && 2 * p.n == p.L;
+    if (!*half && (p.mode == MODE_LAST || p.n != p.L)) return false;
+    const bool stage = p.mode != MODE_LAST && p.inner == 1;
+    *d = p.mode == MODE_LAST ? dft_shape<MODE_LAST>(p.L, p.n, *half, stage) : dft_shape<MODE_MID>(p.L, p.n, *half, stage);
+    return d->smem <= kDftSmem;
+}
+
 template <int MODE, int SRC, bool HALF>
-cudaError_t launch_dft_t(const Pass& p, const PassArgs& a, cudaStream_t st) {
+cudaError_t launch_dft_t(const Pass& p, const PassArgs& a, const DftShape& d, cudaStream_t st) {
     const int64_t lines = MODE == MODE_LAST ? a.S * p.inner : a.S * p.outer * p.inner;
-    if (lines <= 0) return cudaSuccess;
-    const DftShape d = dft_shape<MODE>(p.L, p.n, HALF, MODE != MODE_LAST && p.inner == 1);
-    if (d.smem > kDftSmem) return cudaErrorNotSupported;
     auto k = pass_dft<MODE, SRC, HALF>;
     cudaError_t e = smem_limit_once((const void*)k, d.smem);
     if (e != cudaSuccess) return e;
@@ -404,14 +413,12 @@ cudaError_t launch_direct_t(const Pass& p, const PassArgs& a, cudaStream_t st) {
     const int64_t work = (MODE == MODE_LAST) ? a.S * (int64_t)p.L * p.inner
                                              : a.S * p.outer * (int64_t)p.q_out * p.inner;
     if (work <= 0) return cudaSuccess;
-    constexpr bool FWD = MODE == MODE_MID || MODE == MODE_LAST;
-    if (p.L >= 2 && p.L <= kDftMax) {
-        cudaError_t e = cudaErrorNotSupported;
-        if constexpr (FWD)
-            if (2 * p.n == p.L) e = launch_dft_t<MODE, SRC, true>(p, a, st);
-        if constexpr (MODE != MODE_LAST)
-            if (p.n == p.L) e = launch_dft_t<MODE, SRC, false>(p, a, st);
-        if (e != cudaErrorNotSupported) return e;
+    DftShape d;
+    bool half;
+    if (dft_form(p, &d, &half)) {
+        if constexpr (MODE == MODE_MID || MODE == MODE_LAST)
+            if (half) return launch_dft_t<MODE, SRC, true>(p, a, d, st);
+        if constexpr (MODE != MODE_LAST) return launch_dft_t<MODE, SRC, false>(p, a, d, st);
     }
     const int threads = 256;
     const int64_t blocks = (work + threads - 1) / threads;
@@ -423,6 +430,17 @@ cudaError_t launch_direct_t(const Pass& p, const PassArgs& a, cudaStream_t st) {
 }
 
 }  // namespace
+
+LastShape direct_last_shape(const Pass& p, int64_t cc) {
+    DftShape d;
+    bool half;
+    // a sample takes the time of its n terms and of about 24 for the index; a slice's sums
+    // that of 16 to 24, the kernel that adds them that of 200
+    const double sample = p.n + 24;
+    if (dft_form(p, &d, &half))
+        return {(cc * p.inner + d.lines - 1) / d.lines, std::min(3, (int)(kDftSmem / d.smem)), 24.0 / sample, 200.0 / sample};
+    return {(cc * p.L * p.inner + 255) / 256, 6, 16.0 / sample, 200.0 / sample};
+}
 
 cudaError_t launch_direct(const Pass& p, const PassArgs& a, cudaStream_t st) {
     return dispatch_mode(p.mode, [&](auto M) {

@@ -113,6 +113,16 @@ constexpr int level_last_columns(int L, int64_t inner = 2) {
     return L <= 32 && inner > 1 && inner % 2 == 0 ? (L == 16 && inner >= 512 ? 32 : 256 / L) : 0;
 }
 
+// A LAST pass over some channels: its CTAs and how many an SM holds; and in samples' time
+// of a full GPU, what a slice of the samples costs beside (its sums written and read
+// again) and what the kernel that adds the slices does.
+struct LastShape {
+    int64_t ctas;
+    int per_sm;
+    double fold, launch;
+};
+LastShape direct_last_shape(const Pass& p, int64_t cc);  // KIND_DIRECT
+
 // Resident CTAs per SM of the LAST-mode kernel of a KIND_LEVEL pass.
 cudaError_t level_last_occupancy(const Pass& p, int src_kind, int* blocks_per_sm);
 
