@@ -623,7 +623,7 @@ int choose_slices(const omni_plan* pl, int64_t cc, int64_t tc, int64_t most) {
     const Pass& last = pl->fwd.back();
     LastShape s{cc * pl->last_ctas, pl->last_per_sm, 2.0, 6.0};
     if (last.kind == KIND_REG) s.ctas = (cc * last.inner + 255) / 256;
-    if (last.kind == KIND_DIRECT) s = direct_last_shape(last, cc);
+    if (last.kind == KIND_DIRECT) s = direct_last_shape(last, cc, tc);
     const int64_t slots = pl->sms * s.per_sm;
     const double fold = s.fold * s.ctas / slots;
     double best = 0.9 * (double)(tc * ceil_div(s.ctas, slots));
@@ -940,6 +940,7 @@ omni_status run_chunk(omni_plan* pl, const void* volts, int64_t vc0, int64_t Tsr
         }
         if (p.mode == MODE_LAST) {
             a.S = cc;
+            a.full_S = chunk_channels(pl);
             if (pl->slices > 1 && tc != pl->sliced_tc) {
                 pl->sliced = choose_slices(pl, chunk_channels(pl), tc, pl->slices);
                 pl->sliced_tc = tc;
@@ -948,6 +949,7 @@ omni_status run_chunk(omni_plan* pl, const void* volts, int64_t vc0, int64_t Tsr
             a.part = pl->part;
         } else {
             a.S = cc * tc;
+            a.full_S = chunk_channels(pl) * tc;
             a.dst = dst;
             a.dst_stride = p.outer * p.q_out * p.inner;
         }

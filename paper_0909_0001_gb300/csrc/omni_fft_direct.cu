@@ -1,8 +1,9 @@
 // omni_fft_direct.cu -- direct-DFT axis transforms.
 //
 // Axes of any length (non-powers of two, and the degenerate single-antenna
-// lattice).  Up to kDftMax points, as shared memory allows: tiles of lines in shared memory, sums shared
-// between the outputs of opposite and shifted bins; longer: one thread per output.
+// lattice).  Up to kDftMax points, as shared memory allows, and for enough work: tiles of
+// lines in shared memory, sums shared between the outputs of opposite and shifted bins;
+// else one thread per output.
 #include "omni_fft_common.cuh"
 
 #include <algorithm>
@@ -397,6 +398,19 @@ bool dft_form(const Pass& p, DftShape* d, bool* half) {
     return d->smem <= kDftSmem;
 }
 
+// Whether the tiles take S samples (LAST: channels of tc samples), by the terms that the
+// pass sums: below, their tables and barriers (2 to 4 us) cost more than they save.  By 530
+// passes of 6 to 192 points run in both forms: forward MID passes cross at 2 to 4 M terms
+// (24 points, 0.7 M: 13.4 against 8.3 us; 22 M: 18 against 33), inverse MID ones at 1 to 2 M
+// (longer lines later), the last at 8 M (14 against 12; 41 M: 18 against 35), LAST passes at
+// 2 to 4 M (24 points, 0.9 M: 10.3 against 8.0; 14 M: 13.7 against 22.6).
+bool dft_takes(const Pass& p, int64_t S, int64_t tc, DftShape* d, bool* half) {
+    const bool last = p.mode == MODE_LAST;
+    const double outputs = last ? (double)S * tc * p.L * p.inner : (double)S * p.outer * p.q_out * p.inner;
+    const int least = last ? 3 : p.mode == MODE_INV_LAST ? 8 : 4;
+    return outputs * p.n >= (double)(least << 20) && dft_form(p, d, half);
+}
+
 template <int MODE, int SRC, bool HALF>
 cudaError_t launch_dft_t(const Pass& p, const PassArgs& a, const DftShape& d, cudaStream_t st) {
     const int64_t lines = MODE == MODE_LAST ? a.S * p.inner : a.S * p.outer * p.inner;
@@ -415,7 +429,7 @@ cudaError_t launch_direct_t(const Pass& p, const PassArgs& a, cudaStream_t st) {
     if (work <= 0) return cudaSuccess;
     DftShape d;
     bool half;
-    if (dft_form(p, &d, &half)) {
+    if (dft_takes(p, a.full_S ? a.full_S : a.S, a.tc, &d, &half)) {
         if constexpr (MODE == MODE_MID || MODE == MODE_LAST)
             if (half) return launch_dft_t<MODE, SRC, true>(p, a, d, st);
         if constexpr (MODE != MODE_LAST) return launch_dft_t<MODE, SRC, false>(p, a, d, st);
@@ -431,13 +445,13 @@ cudaError_t launch_direct_t(const Pass& p, const PassArgs& a, cudaStream_t st) {
 
 }  // namespace
 
-LastShape direct_last_shape(const Pass& p, int64_t cc) {
+LastShape direct_last_shape(const Pass& p, int64_t cc, int64_t tc) {
     DftShape d;
     bool half;
     // a sample takes the time of its n terms and of about 24 for the index; a slice's sums
     // that of 16 to 24, the kernel that adds them that of 200
     const double sample = p.n + 24;
-    if (dft_form(p, &d, &half))
+    if (dft_takes(p, cc, tc, &d, &half))
         return {(cc * p.inner + d.lines - 1) / d.lines, std::min(3, (int)(kDftSmem / d.smem)), 24.0 / sample, 200.0 / sample};
     return {(cc * p.L * p.inner + 255) / 256, 6, 16.0 / sample, 200.0 / sample};
 }

@@ -76,6 +76,8 @@ struct PassArgs {
     int64_t T, t0, N;    // voltages: samples per channel row, first sample, antennas
     int tc;              // samples per channel in this chunk
     int64_t S;           // MID/INV: samples (channels) in the launch; LAST: channels
+    int64_t full_S;      // S of a call's full chunks (0: S), by which kernels are chosen: results must
+                         //     not depend on how the channels were cut
     int64_t c0;          // channel of the first sample in P / V
     float2* dst;
     int64_t dst_stride;  // elements per sample of dst
@@ -113,15 +115,15 @@ constexpr int level_last_columns(int L, int64_t inner = 2) {
     return L <= 32 && inner > 1 && inner % 2 == 0 ? (L == 16 && inner >= 512 ? 32 : 256 / L) : 0;
 }
 
-// A LAST pass over some channels: its CTAs and how many an SM holds; and in samples' time
-// of a full GPU, what a slice of the samples costs beside (its sums written and read
+// A LAST pass over some channels and samples: its CTAs and how many an SM holds; and in
+// samples' time of a full GPU, what a slice of the samples costs beside (its sums written and read
 // again) and what the kernel that adds the slices does.
 struct LastShape {
     int64_t ctas;
     int per_sm;
     double fold, launch;
 };
-LastShape direct_last_shape(const Pass& p, int64_t cc);  // KIND_DIRECT
+LastShape direct_last_shape(const Pass& p, int64_t cc, int64_t tc);  // KIND_DIRECT
 
 // Resident CTAs per SM of the LAST-mode kernel of a KIND_LEVEL pass.
 cudaError_t level_last_occupancy(const Pass& p, int src_kind, int* blocks_per_sm);

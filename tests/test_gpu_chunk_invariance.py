@@ -1,7 +1,7 @@
 """The same samples give the same bits however their channels are cut into chunks: host
 input starts with a quarter of a chunk and grows, device input is cut equally.  Shapes
-whose LAST pass is cut into slices (which go by the plan's
-chunk and the samples, not by the piece at hand)."""
+whose LAST pass is cut into slices or whose passes have two forms (slices and forms go by
+the plan's chunk and the samples, not by the piece at hand)."""
 import numpy as np
 import pytest
 import torch
