@@ -185,12 +185,14 @@ __global__ void __launch_bounds__(kFThreads) fengine_fused(const int8_t* __restr
 // 32-byte sector).  Buffer index of point m: 9 (m / 8) + m % 8 and a transform pitch of
 // 72: the half-warps of every step touch 16 different bank pairs.
 // 16384 antennas, 4 taps, 1024 frames, int8 out: 6.33 -> 3.59 ms.
+// PART (up to 28 antennas): warps without an antenna only meet the barriers (8 antennas, 1
+// tap, 2048 frames: 23 -> 12 us; in every group the test costs the large case 6%).
 constexpr int kF64Ant = 32;
 constexpr int kF64Frames = 16;  // most frames per CTA; fewer (even) while the GPU is not filled
 constexpr int kF64MaxTaps = 8;
 constexpr int kF64Row = 36;  // char2 per staged row (72 bytes: conflict-free 2-byte stores and 8-byte loads)
 
-template <bool I8, bool GAINS>
+template <bool I8, bool GAINS, bool PART>
 __global__ void __launch_bounds__(256, 2) fengine64(const int8_t* __restrict__ raw, int64_t N, int64_t S, int P,
                                                     const float* __restrict__ w, int64_t T,
                                                     const float2* __restrict__ gains, float scale,
@@ -207,6 +209,7 @@ __global__ void __launch_bounds__(256, 2) fengine64(const int8_t* __restrict__ r
     const int al = 4 * warp + tr;  // antenna within the CTA
     const int64_t a = a0 + al;
     const int64_t last = a < N ? T + P - 1 : 0;  // frames of this antenna that exist
+    const bool idle = PART && a0 + 4 * warp >= N;  // none of this warp's antennas exists
     float2* buf = zs[warp] + 72 * tr;
     // step-1 twiddles, unpacking twiddles e^{-i pi f / 64} and the gains of this lane's f = l + 8 k_b
     float2 t1[8], ut[8], gl[GAINS ? 8 : 1];
@@ -232,7 +235,7 @@ __global__ void __launch_bounds__(256, 2) fengine64(const int8_t* __restrict__ r
         // polyphase sums of samples 16 l .. 16 l + 15 of frames t and t + 1:
         // z(8 l + q) = u(16 l + 2q) + i u(16 l + 2q + 1)
         float u0[16], u1[16];
-        {
+        if (!idle) {
             float x0[16], x1[16];
 #pragma unroll
             for (int b = 0; b < 16; ++b) u0[b] = u1[b] = 0.f;
@@ -316,8 +319,10 @@ __global__ void __launch_bounds__(256, 2) fengine64(const int8_t* __restrict__ r
                 }
             }
         };
-        transform(u0, 0);
-        transform(u1, 1);
+        if (!idle) {
+            transform(u0, 0);
+            transform(u1, 1);
+        }
         if (I8) {
             // rows (channel f, frame t + fr) of the CTA's 32 antennas, 16 (32 bytes) per thread;
             // the other parity's rows are written next, so one barrier per pair is enough
@@ -329,11 +334,14 @@ __global__ void __launch_bounds__(256, 2) fengine64(const int8_t* __restrict__ r
 #pragma unroll
                 for (int i = 0; i < 4; ++i) c[i] = q[i];
                 char2* o = reinterpret_cast<char2*>(out) + ((int64_t)f * T + t + fr) * N + a0 + h;
-                if (a0 + h + 16 <= N && ((uintptr_t)o % 16) == 0) {
-                    reinterpret_cast<uint4*>(o)[0] = make_uint4(c[0].x, c[0].y, c[1].x, c[1].y);
-                    reinterpret_cast<uint4*>(o)[1] = make_uint4(c[2].x, c[2].y, c[3].x, c[3].y);
-                } else {
-                    for (int k = 0; k < 16 && a0 + h + k < N; ++k) o[k] = yq[par][fr][f][h + k];
+#pragma unroll
+                for (int g = 0; g < 16; g += 8) {
+                    if (a0 + h + g + 8 <= N && ((uintptr_t)(o + g) % 16) == 0) {
+                        const uint2 u = c[g / 4], v = c[g / 4 + 1];
+                        *reinterpret_cast<uint4*>(o + g) = make_uint4(u.x, u.y, v.x, v.y);
+                    } else {
+                        for (int k = g; k < g + 8 && a0 + h + k < N; ++k) o[k] = yq[par][fr][f][h + k];
+                    }
                 }
             }
         }
@@ -686,8 +694,12 @@ cudaError_t launch_fengine(const int8_t* raw, int64_t N, int64_t S, int32_t F, i
         const int64_t groups = (N + kF64Ant - 1) / kF64Ant;
         while (frames > 2 && groups * ((T + frames - 1) / frames) < 152) frames /= 2;
         const unsigned c64 = (unsigned)(groups * ((T + frames - 1) / frames));
-        auto k = out_i8 ? (gains ? fengine64<true, true> : fengine64<true, false>)
-                        : (gains ? fengine64<false, true> : fengine64<false, false>);
+        auto pick = [&](auto part) {
+            constexpr bool PART = decltype(part)::value;
+            return out_i8 ? (gains ? fengine64<true, true, PART> : fengine64<true, false, PART>)
+                          : (gains ? fengine64<false, true, PART> : fengine64<false, false, PART>);
+        };
+        auto k = N <= kF64Ant - 4 ? pick(std::true_type{}) : pick(std::false_type{});
         k<<<c64, 256, 0, st>>>(raw, N, S, P, window, T, gains, scale, out, frames);
         return cudaGetLastError();
     }

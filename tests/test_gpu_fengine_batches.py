@@ -43,6 +43,12 @@ def test_64_channel_frame_runs(N, T, P, gains):
     check(64, N, T, P, 0, gains, list(range(0, N, 37)) + [N - 1])
 
 
+@pytest.mark.parametrize("N, T, P, gains", [(8, 2101, 1, False), (3, 2099, 4, True), (20, 1303, 8, False), (28, 2500, 3, True),
+                                            (40, 1301, 4, False)])
+def test_64_channels_of_a_few_antennas(N, T, P, gains):
+    check(64, N, T, P, 0, gains, [0, N // 2, N - 1])
+
+
 @pytest.mark.parametrize("F, N, T, P, extra, gains", [(16, 300, 261, 4, 0, False), (16, 260, 301, 1, 3, True),
                                                       (32, 200, 197, 5, 1, True), (64, 150, 131, 4, 2, False),
                                                       (128, 70, 141, 3, 0, True), (256, 35, 141, 4, 2, True),
