@@ -386,7 +386,7 @@ __device__ __forceinline__ void dit(float2 (&v)[R], const float2* tw, int pos, i
 // 1000 antennas, 1024 channels, 8 taps, 200 frames, float out: 6.49 (radix-2 passes in shared
 // memory, spectra through a scratch buffer) -> 1.94 ms; 2.36 with four frames and one antenna
 // per thread, two antennas per CTA, and a table without pads.
-template <int LOGF>
+template <int LOGF, bool FEW>
 struct MGeom {
     static constexpr int F = 1 << LOGF;
     static constexpr int R1 = LOGF <= 5 ? 4 : LOGF == 6 || LOGF == 9 ? 8 : 16;
@@ -394,7 +394,7 @@ struct MGeom {
     static constexpr int R2 = F / (R1 * R3);
     static constexpr int R = 2;
     static constexpr int TH = 256;
-    static constexpr int A0 = 8192 / (R * F), A = A0 > 128 ? 128 : A0;
+    static constexpr int A0 = 8192 / (R * F) / (FEW ? 4 : 1), A = A0 > 128 ? 128 : A0 < 1 ? 1 : A0;
     static constexpr int AT = A > 1 ? 2 : 1;                                // antennas per thread, polyphase sums
     static constexpr int RT = A * R1 * R2 / 2 >= TH ? R : 1;                // frames per thread, last step
     static constexpr int P2 = R3 + 1;
@@ -406,13 +406,14 @@ struct MGeom {
     static_assert(SMEM <= 113 * 1024, "two CTAs per SM");
 };
 
-template <int LOGF>
-__global__ void __launch_bounds__(MGeom<LOGF>::TH, 2) fengine_multi(const int8_t* __restrict__ raw, int64_t N, int64_t S,
-                                                                 int P, const float* __restrict__ w, int64_t T,
-                                                                 const float2* __restrict__ gains, float scale,
-                                                                 void* __restrict__ out, int out_i8, int vec,
-                                                                 int batches_per_cta) {
-    using G = MGeom<LOGF>;
+// FEW: a quarter of the antennas per CTA.
+template <int LOGF, bool FEW>
+__global__ void __launch_bounds__(MGeom<LOGF, FEW>::TH, 2) fengine_multi(const int8_t* __restrict__ raw, int64_t N,
+                                                                      int64_t S, int P, const float* __restrict__ w,
+                                                                      int64_t T, const float2* __restrict__ gains,
+                                                                      float scale, void* __restrict__ out, int out_i8,
+                                                                      int vec, int batches_per_cta) {
+    using G = MGeom<LOGF, FEW>;
     constexpr int F = G::F, R1 = G::R1, R2 = G::R2, R3 = G::R3, R = G::R, TH = G::TH, A = G::A, AT = G::AT, RT = G::RT;
     constexpr int P1 = G::P1, P2 = G::P2, PLANE = G::PLANE, H = R1 * R2;
     extern __shared__ float2 sm[];
@@ -620,11 +621,18 @@ __global__ void __launch_bounds__(MGeom<LOGF>::TH, 2) fengine_multi(const int8_t
     }
 }
 
-template <int LOGF>
+template <int LOGF, bool FEW = false>
 cudaError_t launch_multi(const int8_t* raw, int64_t N, int64_t S, int P, const float* w, int64_t T, const float2* gains,
                          float scale, void* out, int out_i8, cudaStream_t st) {
-    using G = MGeom<LOGF>;
-    auto k = fengine_multi<LOGF>;
+    using G = MGeom<LOGF, FEW>;
+    // beyond 256 channels (below, the 16-antenna pass takes the small calls), fewer CTAs than
+    // SMs: a quarter of the antennas each (512 channels, 8 antennas, 4 frames, 12 taps, odd rows:
+    // two CTAs 37.5 us, eight 14)
+    if constexpr (!FEW && LOGF >= 9 && G::A > 1) {
+        if ((N + G::A - 1) / G::A * ((T + G::R - 1) / G::R) < 152)
+            return launch_multi<LOGF, true>(raw, N, S, P, w, T, gains, scale, out, out_i8, st);
+    }
+    auto k = fengine_multi<LOGF, FEW>;
     cudaError_t e = smem_limit_once((const void*)k, G::SMEM);
     if (e != cudaSuccess) return e;
     // 4-byte sample loads and 16-byte window loads where the rows allow them

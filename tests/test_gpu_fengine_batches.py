@@ -61,3 +61,11 @@ def test_16_to_256_channels_on_a_filled_gpu(F, N, T, P, extra, gains):
                                                (512, 100, 401, 4, True), (1024, 39, 489, 1, False)])
 def test_several_batches_per_cta(F, N, T, P, gains):
     check(F, N, T, P, 0, gains, [0, N // 2, N - 1])
+
+
+@pytest.mark.parametrize("F, N, T, P, extra, gains", [(512, 20, 101, 5, 3, True), (1024, 9, 103, 2, 0, False),
+                                                      (2048, 5, 103, 1, 1, True),                      # a CTA per SM
+                                                      (512, 20, 99, 5, 3, True), (1024, 5, 63, 3, 0, True),
+                                                      (2048, 3, 7, 12, 2, False)])                     # fewer
+def test_512_channels_and_more(F, N, T, P, extra, gains):
+    check(F, N, T, P, extra, gains, [0, 1, N - 1])
