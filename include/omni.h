@@ -110,8 +110,9 @@ omni_status omni_baselines(const omni_level* levels, int n_levels, int32_t* dm,
  * prod L_d; mixed plans [C][L1 L2 of level 1][(2 n3 - 1)(2 n4 - 1)] complex),
  * scratch buffers and staging memory; all are allocated here.  The samples of
  * each omni_correlate call are processed in chunks the plan sizes itself (from
- * its buffer target, the kernels' occupancy and, for mixed plans, whole waves
- * of CTAs); results do not depend on the chunking.
+ * its buffer target, halved while the device has less memory left than two
+ * such buffers, the kernels' occupancy and, for mixed plans, whole waves
+ * of CTAs); results do not depend on the chunking beyond rounding.
  * Errors: INVALID_ARG, COLLISION, UNSUPPORTED (more than 8 levels, a padded
  * axis longer than 4096, or a non-power-of-two padded axis longer than 1024;
  * mixed precision outside 2-level hierarchies of at most 64 level-1 blocks

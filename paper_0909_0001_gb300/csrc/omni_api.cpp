@@ -275,6 +275,7 @@ struct omni_plan {
     int* host_err = nullptr;
     int* dev_err = nullptr;   // its device address
     int force_expire = 0;     // OMNI_TEST_FORCE_TIMEOUT: tensor-core waits expire (tests)
+    int no_slices = 0;        // OMNI_TEST_NO_SLICES: no memory for the slices' sums (tests)
     std::vector<float2*> tw_tables;
     // host-input staging
     void* stage[2] = {nullptr, nullptr};
@@ -723,6 +724,31 @@ void choose_chunks(omni_plan* pl) {
     pl->buf_elems = std::max(pl->Cc * pl->Tc * pl->fwd_elems, pl->Cv * pl->inv_elems);
     if (last.kind == KIND_XSPEC5 || last.kind == KIND_COV5)  // the second buffer also holds the transposed accumulator
         pl->buf_elems = std::max(pl->buf_elems, pl->Cv * acc_doubles(pl));
+}
+
+// What a chunk needs beside the accumulator, or nothing and the error.  Without room for
+// the slices' sums the plan runs unsliced.
+cudaError_t allocate_chunk_buffers(omni_plan* pl) {
+    bool data_scale = false;
+    for (const Pass& q : pl->fwd) data_scale = data_scale || (q.scale_n > 0 && !q.bf16);
+    cudaError_t e = data_scale ? cudaMalloc(&pl->chan_max, (size_t)2 * pl->Cc * sizeof(float)) : cudaSuccess;
+    for (int b = 0; b < 2 && e == cudaSuccess; ++b)
+        e = cudaMalloc(&pl->buf[b], (size_t)std::max<int64_t>(1, pl->buf_elems) * sizeof(float2));
+    if (e != cudaSuccess) {
+        cudaFree(pl->chan_max);
+        cudaFree(pl->buf[0]);
+        cudaFree(pl->buf[1]);
+        pl->chan_max = nullptr;
+        pl->buf[0] = pl->buf[1] = nullptr;
+        return e;
+    }
+    const size_t part_bytes = (size_t)pl->slices * pl->Cc * acc_doubles(pl) * sizeof(float);
+    if (pl->slices > 1 && (pl->no_slices || cudaMalloc(&pl->part, part_bytes) != cudaSuccess)) {
+        cudaGetLastError();
+        pl->part = nullptr;
+        pl->slices = 1;
+    }
+    return cudaSuccess;
 }
 
 // After a stream synchronisation: report (and clear) an expired device wait.
@@ -1469,6 +1495,7 @@ static omni_status create_plan(const omni_level* levels, int n_levels, int64_t n
     pl->dtype = dtype;
     pl->precision = precision;
     if (const char* env = std::getenv("OMNI_TEST_FORCE_TIMEOUT")) pl->force_expire = std::atoi(env) != 0;
+    if (const char* env = std::getenv("OMNI_TEST_NO_SLICES")) pl->no_slices = std::atoi(env) != 0;
     cudaError_t e = cudaGetDevice(&pl->device);
     if (e != cudaSuccess) {
         delete pl;
@@ -1552,27 +1579,24 @@ static omni_status create_plan(const omni_level* levels, int n_levels, int64_t n
         cudaGetLastError();
     }
     init_stats(pl);
-    const size_t buf_bytes = (size_t)std::max<int64_t>(1, pl->buf_elems) * sizeof(float2);
     const size_t P_bytes = (size_t)pl->C * acc_doubles(pl) * sizeof(double);
-    bool data_scale = false;
-    for (const Pass& q : pl->fwd) data_scale = data_scale || (q.scale_n > 0 && !q.bf16);
-    if (data_scale && (e = cudaMalloc(&pl->chan_max, (size_t)2 * pl->Cc * sizeof(float))) != cudaSuccess) {
-        release(pl);
-        return cuda_fail(e, "cudaMalloc");
-    }
-    if (pl->slices > 1 &&
-        (e = cudaMalloc(&pl->part, (size_t)pl->slices * pl->Cc * acc_doubles(pl) * sizeof(float))) != cudaSuccess) {
-        release(pl);
-        return cuda_fail(e, "cudaMalloc");
-    }
-    if ((e = cudaMalloc(&pl->buf[0], buf_bytes)) != cudaSuccess ||
-        (e = cudaMalloc(&pl->buf[1], buf_bytes)) != cudaSuccess ||
-        (e = cudaMalloc(&pl->P, P_bytes)) != cudaSuccess ||
+    if ((e = cudaMalloc(&pl->P, P_bytes)) != cudaSuccess ||
         (e = cudaMemset(pl->P, 0, P_bytes)) != cudaSuccess ||
         (e = cudaHostAlloc(reinterpret_cast<void**>(&pl->host_err), sizeof(int), cudaHostAllocMapped)) != cudaSuccess ||
         (e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&pl->dev_err), pl->host_err, 0)) != cudaSuccess) {
         release(pl);
         return cuda_fail(e, "allocating plan buffers");
+    }
+    // less device memory left than the chunks take: smaller chunks (FP32 tile plans once took
+    // one channel of samples, and run with that still)
+    while ((e = allocate_chunk_buffers(pl)) == cudaErrorMemoryAllocation && pl->knobs.chunk_mb > 1) {
+        cudaGetLastError();
+        pl->knobs.chunk_mb /= 2;
+        choose_chunks(pl);
+    }
+    if (e != cudaSuccess) {
+        release(pl);
+        return cuda_fail(e, "cudaMalloc");
     }
     *pl->host_err = 0;
     *out = pl;
