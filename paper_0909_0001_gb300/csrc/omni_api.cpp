@@ -882,8 +882,8 @@ double pass_flops(const Pass& p, const PassArgs& a) {
     const double lg = std::log2((double)std::max(p.L, 2));
     const double line = 5.0 * p.L * lg;
     switch (p.kind) {
-        case KIND_XSPEC:  // one complex multiply-add per tile pair, frequency and sample
-            return (double)a.S * a.tc * p.outer * p.outer * p.L * 8.0;
+        case KIND_XSPEC:  // one complex multiply-add per tile pair (each once), frequency and sample
+            return (double)a.S * a.tc * 0.5 * p.outer * (p.outer + 1) * p.L * 8.0;
         case KIND_COV5:
         case KIND_XSPEC5:  // the same products in real form: 3 (FP16 split) or 6 (BF16) x (2 n_tiles)^2 MACs
             return (double)a.S * a.tc * p.L * (p.bf16 ? 6.0 : 3.0) * (2.0 * p.outer) * (2.0 * p.outer) * 2.0;

@@ -1,0 +1,26 @@
+"""The statistics of a plan's kernels: what they say of launches, bytes and operations is
+what the kernels that ran do."""
+import pytest
+
+from paper_0909_0001_gb300 import omni, synth
+
+pytestmark = pytest.mark.gpu
+
+
+def stats_of(plan, x):
+    plan.kernel_stats(clear=True)
+    plan.profile(True)
+    plan.correlate(x)
+    plan.visibilities()
+    plan.profile(False)
+    return {s["name"]: s for s in plan.kernel_stats(clear=True)}
+
+
+def test_fp32_tile_pairs_count_each_pair_once():
+    n, C, T, K = 20, 2, 7, 16
+    x = synth.random_complex([2, 2, n], C, T, seed=1800)
+    with omni.TilePlan(synth.Level(2, 2), [(10.0 * i, 0.0) for i in range(n)], C) as plan:
+        s = stats_of(plan, x.cuda())
+    xspec = [v for k, v in s.items() if "xspec" in k]
+    assert len(xspec) == 1 and xspec[0]["launches"] == 1
+    assert xspec[0]["flops"] == 8.0 * C * T * K * n * (n + 1) / 2
