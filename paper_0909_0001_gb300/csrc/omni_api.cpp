@@ -902,7 +902,7 @@ double pass_flops(const Pass& p, const PassArgs& a) {
             const double lines = (p.mode == MODE_LAST) ? (double)a.S * a.tc * p.inner
                                                        : (double)a.S * p.outer * p.inner;
             const double extra = (p.mode == MODE_LAST) ? 3.0 * p.L : 0.0;
-            const double per = p.kind == KIND_DIRECT ? 8.0 * p.n * p.q_out : line;
+            const double per = p.kind == KIND_DIRECT ? direct_line_flops(p, a) : line;
             return lines * (per + extra);
         }
     }

@@ -456,6 +456,14 @@ LastShape direct_last_shape(const Pass& p, int64_t cc, int64_t tc) {
     return {(cc * p.L * p.inner + 255) / 256, 6, 16.0 / sample, 200.0 / sample};
 }
 
+double direct_line_flops(const Pass& p, const PassArgs& a) {
+    DftShape d;
+    bool half;
+    // tiles: four real multiply-adds per term and bin r give two or four outputs
+    if (dft_takes(p, a.full_S ? a.full_S : a.S, a.tc, &d, &half)) return 8.0 * d.rows * d.reps;
+    return 8.0 * p.n * p.q_out;
+}
+
 cudaError_t launch_direct(const Pass& p, const PassArgs& a, cudaStream_t st) {
     return dispatch_mode(p.mode, [&](auto M) {
         return dispatch_src<decltype(M)::value>(a.src_kind, [&](auto S) {

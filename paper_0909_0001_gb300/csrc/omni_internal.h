@@ -125,6 +125,9 @@ struct LastShape {
 };
 LastShape direct_last_shape(const Pass& p, int64_t cc, int64_t tc);  // KIND_DIRECT
 
+// Operations on one line of a KIND_DIRECT launch, by the form that takes it.
+double direct_line_flops(const Pass& p, const PassArgs& a);
+
 // Resident CTAs per SM of the LAST-mode kernel of a KIND_LEVEL pass.
 cudaError_t level_last_occupancy(const Pass& p, int src_kind, int* blocks_per_sm);
 

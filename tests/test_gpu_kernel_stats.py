@@ -24,3 +24,13 @@ def test_fp32_tile_pairs_count_each_pair_once():
     xspec = [v for k, v in s.items() if "xspec" in k]
     assert len(xspec) == 1 and xspec[0]["launches"] == 1
     assert xspec[0]["flops"] == 8.0 * C * T * K * n * (n + 1) / 2
+
+
+@pytest.mark.parametrize("C, T, per_line", [(28, 110, 8 * 12 * 7), (1, 3, 8 * 12 * 24)])  # tiles of lines; per output
+def test_direct_passes_count_what_their_form_sums(C, T, per_line):
+    x = synth.random_complex([2, 12], C, T, seed=1801)
+    with omni.Plan([synth.Level(2, 12)], C) as plan:
+        s = stats_of(plan, x.cuda())
+    last = [v for k, v in s.items() if k.startswith("fwd axis1 direct24 last")]
+    assert len(last) == 1
+    assert last[0]["flops"] == C * T * 4 * (per_line + 3 * 24)
