@@ -157,7 +157,7 @@ _PASS_SOURCES = [("lagsum-tcgen05", ("omni_xspec5.cu",)), ("xspec-tcgen05", ("om
                  ("smem", ("omni_fft_smem.cuh", "omni_fft_smem_a.cu", "omni_fft_smem_b.cu",
                            "omni_fft_smem_c.cu")),
                  ("reg", ("omni_fft_reg.cuh", "omni_fft_reg_a.cu", "omni_fft_reg_b.cu")),
-                 ("direct", ("omni_fft_direct.cu",))]
+                 ("direct", ("omni_fft_direct.cu",)), ("fold", ("omni_fold.cu",))]
 
 
 def kernel_source_hash(pass_name):

@@ -280,13 +280,15 @@ typedef struct omni_kernel_stat {
                           outputs written at their stored precision */
     double flops;      /* algorithmic floating-point operations of all launches:
                           5 L log2 L per L-point line transform plus 3 per |F|^2
-                          term for the FFT passes; the executed m16n8k16 products
-                          (4096 each) for the tensor-core passes */
+                          term for the FFT passes; the multiply-adds executed for
+                          direct DFTs and FP32 tile pairs (each pair once) and the
+                          m16n8k16 products (4096 each) for the tensor-core passes */
     int32_t tensor;    /* 1 when the pass runs on tensor cores */
 } omni_kernel_stat;
 
 /* Start (enable != 0) or stop recording a CUDA event pair around every kernel
- * launch of the plan.  Launch counts are kept whether or not profiling is on. */
+ * launch of the plan's passes (a last pass cut into slices of the samples has a
+ * second entry for the kernel that adds them, "... fold last").  Launch counts are kept whether or not profiling is on. */
 omni_status omni_profile_enable(omni_plan* plan, int enable);
 
 /* Copy up to max per-pass statistics into out (n_out receives how many);

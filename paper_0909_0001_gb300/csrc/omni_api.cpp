@@ -836,6 +836,11 @@ void init_stats(omni_plan* pl) {
                  pl->split_pass.axis + 1, pl->split_pass.L);
         pl->stats.push_back(st);
     }
+    if (pl->slices > 1) {  // the sums of the last pass's slices
+        omni_kernel_stat st{};
+        snprintf(st.name, sizeof st.name, "fwd axis%d fold last", pl->fwd.back().axis);
+        pl->stats.push_back(st);
+    }
 }
 
 cudaEvent_t pool_event(omni_plan* pl) {
@@ -869,7 +874,8 @@ double pass_bytes(const Pass& p, const PassArgs& a) {
         case MODE_MID:
             return (double)a.S * p.outer * p.inner * (n_in * in + p.q_out * 8.0);
         case MODE_LAST:
-            return (double)a.S * a.tc * p.inner * n_in * in + (double)a.S * p.q_out * p.inner * 16.0;
+            return (double)a.S * a.tc * p.inner * n_in * in +
+                   (double)a.S * p.q_out * p.inner * (a.split > 1 ? 4.0 * a.split : 16.0);
         case MODE_INV_MID:
             return (double)a.S * p.outer * p.inner * (p.n * in + p.q_out * 8.0);
         default:
@@ -908,21 +914,27 @@ double pass_flops(const Pass& p, const PassArgs& a) {
     }
 }
 
-// Launch pass number idx (index into stats) with optional event timing.
-cudaError_t launch_counted(omni_plan* pl, int idx, const Pass& p, const PassArgs& a,
-                           cudaStream_t st) {
+// One launch counted in stats entry idx, with optional event timing.
+template <class F>
+cudaError_t counted(omni_plan* pl, int idx, double bytes, double flops, cudaStream_t st, F&& launch) {
     omni_kernel_stat& s = pl->stats[idx];
     s.launches += 1;
-    s.bytes += pass_bytes(p, a);
-    s.flops += pass_flops(p, a);
-    if (!pl->profiling) return launch_pass(p, a, st);
+    s.bytes += bytes;
+    s.flops += flops;
+    if (!pl->profiling) return launch();
     cudaEvent_t e0 = pool_event(pl), e1 = pool_event(pl);
     if (!e0 || !e1) return cudaErrorMemoryAllocation;
     cudaEventRecord(e0, st);
-    cudaError_t e = launch_pass(p, a, st);
+    cudaError_t e = launch();
     cudaEventRecord(e1, st);
     pl->pending.push_back({idx, e0, e1});
     return e;
+}
+
+// Launch pass number idx (index into stats).
+cudaError_t launch_counted(omni_plan* pl, int idx, const Pass& p, const PassArgs& a,
+                           cudaStream_t st) {
+    return counted(pl, idx, pass_bytes(p, a), pass_flops(p, a), st, [&] { return launch_pass(p, a, st); });
 }
 
 // One chunk of forward passes: channels [c0, c0+cc) x samples [t0, t0+tc).
@@ -1000,7 +1012,12 @@ omni_status run_chunk(omni_plan* pl, const void* volts, int64_t vc0, int64_t Tsr
             OMNI_CUDA(cudaEventRecord(pl->split_done[slot], pl->split_stream), "cudaEventRecord");
         }
         cudaError_t e = launch_counted(pl, (int)k, p, a, launch_stream);
-        if (e == cudaSuccess && p.mode == MODE_LAST) e = launch_fold_parts(a, launch_stream);
+        if (e == cudaSuccess && p.mode == MODE_LAST && a.split > 1) {
+            // the slices' sums (the last entry of the statistics), read with the accumulator
+            const double points = (double)a.S * a.P_stride;
+            e = counted(pl, (int)pl->stats.size() - 1, points * (4.0 * a.split + 16.0), points * a.split, launch_stream,
+                        [&] { return launch_fold_parts(a, launch_stream); });
+        }
         if (e != cudaSuccess) return cuda_fail(e, "forward pass launch");
         if (cc_split > 0)
             OMNI_CUDA(cudaStreamWaitEvent(st, pl->split_done[slot], 0), "cudaStreamWaitEvent");
@@ -1578,7 +1595,6 @@ static omni_status create_plan(const omni_level* levels, int n_levels, int64_t n
             p.grid_cap = per_sm * sms;
         cudaGetLastError();
     }
-    init_stats(pl);
     const size_t P_bytes = (size_t)pl->C * acc_doubles(pl) * sizeof(double);
     if ((e = cudaMalloc(&pl->P, P_bytes)) != cudaSuccess ||
         (e = cudaMemset(pl->P, 0, P_bytes)) != cudaSuccess ||
@@ -1598,6 +1614,7 @@ static omni_status create_plan(const omni_level* levels, int n_levels, int64_t n
         release(pl);
         return cuda_fail(e, "cudaMalloc");
     }
+    init_stats(pl);
     *pl->host_err = 0;
     *out = pl;
     return OMNI_OK;

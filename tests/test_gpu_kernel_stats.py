@@ -34,3 +34,26 @@ def test_direct_passes_count_what_their_form_sums(C, T, per_line):
     last = [v for k, v in s.items() if k.startswith("fwd axis1 direct24 last")]
     assert len(last) == 1
     assert last[0]["flops"] == C * T * 4 * (per_line + 3 * 24)
+
+
+def test_slices_of_the_last_pass_and_their_fold():
+    """One 16 x 16 array, 64 samples: the LAST pass writes each slice's FP32 sums, the fold
+    reads them and the FP64 accumulator and writes that."""
+    x = synth.random_complex([16, 16], 1, 64, seed=1802)
+    with omni.Plan([synth.Level(16, 16)], 1) as plan:
+        s = stats_of(plan, x.cuda())
+    last = [v for k, v in s.items() if k.startswith("fwd axis0+1 level32 last")]
+    fold = [v for k, v in s.items() if " fold " in k]
+    assert len(last) == len(fold) == 1
+    assert last[0]["launches"] == fold[0]["launches"] == 1
+    assert fold[0]["total_ms"] > 0 and last[0]["total_ms"] > 0
+    sums = fold[0]["bytes"] - 16 * 1024             # the slices' sums, 4 bytes a point
+    assert sums > 0 and sums % (4 * 1024) == 0
+    assert last[0]["bytes"] == 64 * 256 * 8 + sums
+
+
+def test_unsliced_passes_have_no_fold():
+    x = synth.random_complex([16, 16], 700, 2, seed=1803)
+    with omni.Plan([synth.Level(16, 16)], 700) as plan:
+        s = stats_of(plan, x.cuda())
+    assert not any(" fold " in k and v["launches"] for k, v in s.items())
