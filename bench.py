@@ -214,6 +214,12 @@ def alu_peak_tflops(sm_mhz):
     return 152 * 128 * 2 * sm_mhz * 1e6 / 1e12
 
 
+def fengine_bytes(samples, codes):
+    """(algorithmic, design) bytes of an F-engine call with int8 output: raw samples in
+    and codes out, in one pass at any number of channels."""
+    return samples + codes, samples + codes
+
+
 def units_per_launch(stat, profiled_units):
     """Channel-samples one launch of a forward pass processes (profiled_units:
     channels x samples over all the profiled steps)."""
@@ -746,8 +752,7 @@ def run_ours(args):
         e1.record(stream)
         torch.cuda.synchronize()
         ms_f = e0.elapsed_time(e1) / reps
-        alg = raw.numel() + fout.numel()                  # raw in, int8 voltages out
-        design = alg + 2 * need                           # plus the FP32 spectra round trip
+        alg, design = fengine_bytes(raw.numel(), fout.numel())
         fe = {"value": w.n_antennas * T * F / (ms_f * 1e-3), "unit": UNIT, "ms_per_step": ms_f,
               "channels": F, "taps": P, "frames": T, "antennas": w.n_antennas,
               "hbm": {"algorithmic_bytes": alg, "design_bytes": design,
