@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(kXThreads, 1) xspec5(Pass p, PassArgs a, const
             // the raw values have been consumed (split and stored) and the operand
             // stores are ordered before the MMAs' and the next box's asynchronous
             // accesses: release both
-            asm volatile("fence.proxy.async.shared::cta;");
+            fence_async_smem();
             mbar_arrive(&full[st]);
             mbar_arrive(&raw_empty[rs]);
         }
