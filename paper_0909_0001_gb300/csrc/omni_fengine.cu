@@ -386,6 +386,7 @@ __device__ __forceinline__ void dit(float2 (&v)[R], const float2* tw, int pos, i
 // 1000 antennas, 1024 channels, 8 taps, 200 frames, float out: 6.49 (radix-2 passes in shared
 // memory, spectra through a scratch buffer) -> 1.94 ms; 2.36 with four frames and one antenna
 // per thread, two antennas per CTA, and a table without pads.
+// (256 and 4096 channels spill 72 and 88 bytes at the 128 registers of two CTAs per SM.)
 template <int LOGF, bool FEW>
 struct MGeom {
     static constexpr int F = 1 << LOGF;

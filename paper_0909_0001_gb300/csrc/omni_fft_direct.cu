@@ -125,7 +125,8 @@ __global__ void __launch_bounds__(256) pass_direct(Pass p, PassArgs a) {
 // row table bounds the length: kDftMax points, 41 KB.
 // 50 tiles of 12 x 12 (24-point axes), 16 channels x 500 samples: 1.62 + 4.23 -> 0.50 + 0.71 ms
 // forward, 1.70 + 0.41 -> 0.19 + 0.21 ms inverse (2.7 and 3.9 TB/s; eight loads in flight per
-// thread: with one, 0.70 + 1.30 ms).
+// thread: with one, 0.70 + 1.30 ms).  Padded MID and LAST forms spill 44 and 48 bytes at the
+// 80 registers of three CTAs per SM.
 constexpr int kDftMax = 192;
 constexpr int kDftBins = 4;  // bins r per thread
 constexpr size_t kDftSmem = 224 * 1024;  // whole lines reach it at about 160 points

@@ -23,13 +23,14 @@
 // buffer while the current sample runs steps 2 and 3.  Lines are W consecutive inner
 // indices (strided axes), or, for an axis that is innermost in memory, W consecutive
 // outer lines read and written contiguously: step 1 takes its inputs from memory and step 3,
-// whose bins are consecutive across a warp, writes its outputs there.  LAST keeps |X|^2 of the chunk's samples in registers and
-// folds them into the FP64 accumulator once.  The forward inputs j >= L/2 are zero
-// (padding): step 1 never reads them.
-// What bounds it is shared memory (four 8-byte passes per point and line) and FP32.  1024 x 1024 antennas (2048-point axes),
-// 64 samples, line by line at 512 (LAST 256) threads against pairs, serial:
-// MID 0.48 -> 0.30 ms (5.4 TB/s), LAST 0.65 -> 0.52 ms (inputs and outputs through shared memory
-// too, in pairs: 0.42 and 0.63).
+// whose bins are consecutive across a warp, writes its outputs there.  LAST keeps |X|^2 of
+// the chunk's samples in registers and folds them into the FP64 accumulator once.  The
+// forward inputs j >= L/2 are zero (padding): step 1 never reads them.
+// What bounds it is shared memory (four 8-byte passes per point and line) and FP32.  1024 x
+// 1024 antennas (2048-point axes), 64 samples, line by line at 512 (LAST 256) threads against
+// pairs, serial: MID 0.48 -> 0.30 ms (5.4 TB/s), LAST 0.65 -> 0.59 ms (inputs and outputs
+// through shared memory too, in pairs: MID 0.42).  The 4096-point LAST pass spills 56 bytes
+// at the 128 registers of two CTAs per SM.
 #include "omni_fft_common.cuh"
 
 namespace omni {
