@@ -627,10 +627,11 @@ cudaError_t launch_multi(const int8_t* raw, int64_t N, int64_t S, int P, const f
                          float scale, void* out, int out_i8, cudaStream_t st) {
     using G = MGeom<LOGF, FEW>;
     // beyond 256 channels (below, the 16-antenna pass takes the small calls), fewer CTAs than
-    // SMs: a quarter of the antennas each (512 channels, 8 antennas, 4 frames, 12 taps, odd rows:
-    // two CTAs 37.5 us, eight 14)
+    // a quarter of the SMs: a quarter of the antennas each (512 channels, 8 antennas, 4 frames,
+    // 12 taps, odd rows: two CTAs 37.5 us, eight 14; but 1024 channels, 4 antennas, 256 frames,
+    // 1 tap: 128 CTAs 15 us, 512 21)
     if constexpr (!FEW && LOGF >= 9 && G::A > 1) {
-        if ((N + G::A - 1) / G::A * ((T + G::R - 1) / G::R) < 152)
+        if (4 * ((N + G::A - 1) / G::A) * ((T + G::R - 1) / G::R) < 152)
             return launch_multi<LOGF, true>(raw, N, S, P, w, T, gains, scale, out, out_i8, st);
     }
     auto k = fengine_multi<LOGF, FEW>;

@@ -64,8 +64,8 @@ def test_several_batches_per_cta(F, N, T, P, gains):
 
 
 @pytest.mark.parametrize("F, N, T, P, extra, gains", [(512, 20, 101, 5, 3, True), (1024, 9, 103, 2, 0, False),
-                                                      (2048, 5, 103, 1, 1, True),                      # a CTA per SM
-                                                      (512, 20, 99, 5, 3, True), (1024, 5, 63, 3, 0, True),
-                                                      (2048, 3, 7, 12, 2, False)])                     # fewer
+                                                      (2048, 5, 103, 1, 1, True), (512, 20, 30, 3, 0, False),
+                                                      (512, 13, 23, 5, 3, True), (1024, 5, 33, 3, 0, True),  # a quarter
+                                                      (2048, 3, 7, 12, 2, False)])                           # each
 def test_512_channels_and_more(F, N, T, P, extra, gains):
     check(F, N, T, P, extra, gains, [0, 1, N - 1])
