@@ -615,23 +615,44 @@ omni_status build_passes(omni_plan* pl) {
 int64_t chunk_channels(const omni_plan* pl) { return ceil_div(pl->C, ceil_div(pl->C, pl->Cc)); }
 
 // Slices of the last pass's tc samples over cc channels: too few CTAs leave the GPU
-// idle, but each slice's sums are written and read again (FFT passes: 8 bytes per point of
-// the lattice, where a sample reads 2 to 4, two samples' time) and one more kernel adds
-// them (six).  The number of least time in whole waves, if a tenth less than unsliced.
+// idle, but each slice's sums are written and read again (8 bytes per point of the lattice,
+// two samples' time of the passes that HBM bounds, where a sample reads 2 to 4; less of the
+// others') and one more kernel adds them (3 us and 0.1 a slice: samples by what one takes a
+// CTA, from 0.5 us of 4 and 8 points to 6 of 64).  More slices while each step gains a
+// thirtieth in whole waves, if a twentieth less than unsliced; register passes and 8-point
+// levels fill the memory's bandwidth with half their slots.
 // With a slice's cost taken as a 50th of the pass whatever its samples: three levels of 8 x 8,
-// 8 x 8 and 2 x 2, 16 channels x 4 samples, 1.01 ms a pass, unsliced 0.68.
+// 8 x 8 and 2 x 2, 16 channels x 4 samples, 1.01 ms a pass, unsliced 0.62.  With two samples
+// and six for every kernel: 32 x 32, 16 channels x 4, 103 us, in slices 86.
 int choose_slices(const omni_plan* pl, int64_t cc, int64_t tc, int64_t most) {
     const Pass& last = pl->fwd.back();
     LastShape s{cc * pl->last_ctas, pl->last_per_sm, 2.0, 6.0};
-    if (last.kind == KIND_REG) s.ctas = (cc * last.inner + 255) / 256;
-    if (last.kind == KIND_DIRECT) s = direct_last_shape(last, cc, tc);
+    double most_waves = 2.0;
+    if (last.kind == KIND_REG) {
+        s.ctas = (cc * last.inner + 255) / 256;
+        s.per_sm = last.L <= 8 ? 6 : last.L == 16 ? 4 : last.L == 32 ? 2 : 1;
+        if (last.L >= 32) s.launch = 4.0;
+        most_waves = 0.5;
+    } else if (last.kind == KIND_LEVEL) {
+        if (last.L == 8) most_waves = 0.5;
+        if (last.L == 16) s.launch = 4.0;
+        if (last.L == 32) s.launch = 2.7;
+        if (last.L == 64) s.fold = 0.8, s.launch = 0.5;
+    } else if (last.kind == KIND_SMEM || last.kind == KIND_SMEM3) {
+        s.fold = 0.4;
+        s.launch = last.kind == KIND_SMEM ? 1.5 : 0.6;
+    } else if (last.kind == KIND_DIRECT) {
+        s = direct_last_shape(last, cc, tc);
+        most_waves = 8.0;
+    }
     const int64_t slots = pl->sms * s.per_sm;
-    const double fold = s.fold * s.ctas / slots;
-    double best = 0.9 * (double)(tc * ceil_div(s.ctas, slots));
+    if (s.ctas >= most_waves * slots) return 1;
+    const double fold = s.fold * s.ctas / slots + s.launch / 30.0;
+    double best = 0.95 * (double)(tc * ceil_div(s.ctas, slots));
     int slices = 1;
-    for (int64_t k = 2; k <= std::min(most, tc) && s.ctas < 2 * slots && fold * k + s.launch < best; ++k) {
+    for (int64_t k = 2; k <= std::min(most, tc) && fold * k + s.launch < best; ++k) {
         const double t = (double)(ceil_div(tc, k) * ceil_div(s.ctas * k, slots)) + fold * k + s.launch;
-        if (t < best) best = t, slices = (int)k;
+        if (t < (slices > 1 ? 29.0 / 30.0 : 1.0) * best) best = t, slices = (int)k;
     }
     return slices;
 }

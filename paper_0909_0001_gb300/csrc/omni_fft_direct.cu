@@ -450,11 +450,11 @@ LastShape direct_last_shape(const Pass& p, int64_t cc, int64_t tc) {
     DftShape d;
     bool half;
     // a sample takes the time of its n terms and of about 24 for the index; a slice's sums
-    // that of 16 to 24, the kernel that adds them that of 200
+    // that of 16 to 24, the kernel that adds them that of 150
     const double sample = p.n + 24;
     if (dft_takes(p, cc, tc, &d, &half))
-        return {(cc * p.inner + d.lines - 1) / d.lines, std::min(3, (int)(kDftSmem / d.smem)), 24.0 / sample, 200.0 / sample};
-    return {(cc * p.L * p.inner + 255) / 256, 6, 16.0 / sample, 200.0 / sample};
+        return {(cc * p.inner + d.lines - 1) / d.lines, std::min(3, (int)(kDftSmem / d.smem)), 24.0 / sample, 150.0 / sample};
+    return {(cc * p.L * p.inner + 255) / 256, 6, 16.0 / sample, 150.0 / sample};
 }
 
 double direct_line_flops(const Pass& p, const PassArgs& a) {
