@@ -288,7 +288,8 @@ typedef struct omni_kernel_stat {
 
 /* Start (enable != 0) or stop recording a CUDA event pair around every kernel
  * launch of the plan's passes (a last pass cut into slices of the samples has a
- * second entry for the kernel that adds them, "... fold last").  Launch counts are kept whether or not profiling is on. */
+ * second entry for the kernel that adds them, "... fold last").  Launch counts are
+ * kept whether or not profiling is on. */
 omni_status omni_profile_enable(omni_plan* plan, int enable);
 
 /* Copy up to max per-pass statistics into out (n_out receives how many);
